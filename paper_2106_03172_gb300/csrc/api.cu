@@ -136,6 +136,8 @@ FwdArgs fwd_args(const pet_plan *pl, const float *img, int subset, bool natural)
     a.ny = pl->ny;
     a.nz = sino_inner(pl);
     a.nb = pl->nb;
+    a.nb_mul = pl->nb_mul;
+    a.nb_shift = pl->nb_shift;
     a.layers = pl->layers;
     a.lz = pl->d_lz;
     a.img = img;
@@ -180,8 +182,13 @@ pet_status ratio_subset(const pet_problem *p, const float *f, int t, float *rati
     return launch_forward(a, FWD_RATIO, false, choose_group(pl), s, nullptr);
 }
 
+// Whether a state's projections keep the reference rounding (kRefRounding).
+int ref_rounding(const pet_state *st) {
+    return st->algo == PET_ALGO_SAGA && st->table_dtype == PET_TABLE_BF16 ? 1 : 0;
+}
+
 // Full-data ratio in subset-major order into `ratio` (M * nz).
-pet_status ratio_all(const pet_problem *p, const float *f, float *ratio, cudaStream_t s) {
+pet_status ratio_all(const pet_problem *p, const float *f, float *ratio, cudaStream_t s, int ref = 0) {
     const pet_plan *pl = p->plan;
     FwdArgs a = fwd_args(pl, f, -1, false);
     a.g = p->d_g;
@@ -189,6 +196,7 @@ pet_status ratio_all(const pet_problem *p, const float *f, float *ratio, cudaStr
     a.w_scalar = p->w_scalar;
     a.out = ratio;
     a.status = p->d_status;
+    a.ref = ref;
     return launch_forward(a, FWD_RATIO, false, full_group(pl), s, nullptr);
 }
 
@@ -270,7 +278,7 @@ pet_status state_init(pet_state *st, cudaStream_t s) {
     }
     if (st->algo != PET_ALGO_SAGA) return PET_OK;
     // table q_t = grad Phi_t(f^(0)) for all t, then qbar and d
-    PET_TRY(ratio_all(p, st->img, p->d_ratio, s));
+    PET_TRY(ratio_all(p, st->img, p->d_ratio, s, ref_rounding(st)));
     BackArgs b = back_args(pl, p->d_ratio, -1, false);
     b.t0 = 0;
     b.r_view0 = 0;
@@ -418,6 +426,7 @@ pet_status pet_plan_create(const pet_geometry *g, const pet_subsets *sub, pet_pl
     pl->pairs = pairs;
     pl->na = g->n_angles;
     pl->nb = g->n_bins;
+    bins_division(pl->nb, pl->nb_mul, pl->nb_shift);
     pl->ns = sub->n_subsets;
     pl->N = (int)N;
     pl->M = (int)M;
@@ -448,6 +457,7 @@ pet_status pet_plan_create(const pet_geometry *g, const pet_subsets *sub, pet_pl
         vp.K = (float)(ds / (cm * d));
         vp.invK = (float)(cm * d / ds);
         vp.inv_du = cn != 0.0 ? (float)(-cm / cn) : 0.0f;
+        vp.inv_adu = cn != 0.0 ? (float)std::fabs(cm / cn) : kAxisInv;
         const double off = (n_minor % 2) ? 0.5 : 0.0;
         for (int j = 0; j < pl->nb; ++j) {
             const double sj = ((double)j - 0.5 * (pl->nb - 1)) * ds;
@@ -936,6 +946,7 @@ pet_status enqueue_update(pet_state *st, int algo, const int *t_dev, const float
     a.w_scalar = p->w_scalar;
     a.out = st->ratio;
     a.status = p->d_status;
+    a.ref = ref_rounding(st);
     PET_TRY(launch_forward(a, FWD_RATIO, false, choose_group(pl), s, nullptr, max_sub_rays(pl)));
     BackArgs b = back_args(pl, st->ratio, 0, false);
     b.t_dev = t_dev;
@@ -1827,6 +1838,8 @@ void fill_member(BatchMember &m, const pet_state *st, float alpha, const int *se
     m.nx = pl->nx;
     m.ny = pl->ny;
     m.nb = pl->nb;
+    m.nb_mul = pl->nb_mul;
+    m.nb_shift = pl->nb_shift;
     m.ns = pl->ns;
     m.sens_t = pl->d_sens_t;
     m.sens = pl->d_sens;
@@ -1839,6 +1852,7 @@ void fill_member(BatchMember &m, const pet_state *st, float alpha, const int *se
     m.status = p->d_status;
     m.algo = st->algo;
     m.table_dtype = st->table_dtype;
+    m.ref = ref_rounding(st);
     m.img = st->img;
     m.alt = st->alt;
     m.ratio = st->ratio;

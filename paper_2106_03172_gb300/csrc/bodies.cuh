@@ -27,14 +27,142 @@ constexpr int kTileBlockMax = 1024; // threads of a tile block: kTile * kTile / 
 constexpr int kPersistentBackMax = 256;
 constexpr int kPersistentBackRegs = 48;  // five 256-thread blocks per SM
 
+// The bands [kb, ke) of one ray from this thread, every fourth one from kb on:
+// sum of share times pixel, in units of the ray length per band.
+//
+// A band costs ~16 instructions: its lower end from the batch's base by one
+// FMA, the floor by a directed-rounding add (kRound), the share by one
+// saturating multiply, then two loads and three FMAs.  256^2, ncu: a full ratio
+// pass 23.2 us and 14.4M warp instructions (33.2 us and 22.0M with floorf, the
+// comparison of both band ends and contiguous bands per lane), a subset pass
+// 6.9 us (7.9).
+template <bool COH>
+__device__ __forceinline__ float walk_bands(const FwdArgs &a, const ViewParams &vp, float uf, int ui, float hm,
+                                            int n_minor, int kb, int ke) {
+    const int s_major = vp.col ? 1 : a.nx;
+    const int s_minor = vp.col ? a.nx : 1;
+    const float *img1 = a.img + s_minor;
+    // the band's lower end is at its far boundary when the line moves down
+    const float k_end = (vp.du < 0.0f ? 1.0f : 0.0f) - hm;
+    float acc = 0.0f;
+    // kBatch bands at a time: all their offsets and shares first, then the
+    // loads, then the FMAs in band order, so that the loads of a batch are in
+    // flight together.
+    constexpr int kBatch = 4;
+    for (int k = kb; k < ke; k += 4 * kBatch) {
+        // the batch's base position: the integer part of kc du goes into the
+        // pixel index, so that what is left stays small and exact
+        const float kc = (float)k + k_end;
+        const float tp = fmaf(kc, vp.du, kRound);
+        const float base = uf + fmaf(kc, vp.du_lo, fmaf(kc, vp.du, kRound - tp));
+        const unsigned iu = (unsigned)ui + __float_as_uint(tp) - 2u * kRoundBits;
+        int m0[kBatch];
+        float c0[kBatch];
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b) {
+            const float lo = fmaf(4.0f * (float)b, vp.du, base);
+            const float t = __fadd_rd(lo, kRound);
+            m0[b] = (int)(__float_as_uint(t) + iu);
+            c0[b] = band_share(t - (kRound - 1.0f), lo, vp.inv_adu);
+        }
+        // a piece outside the image (or of a band past ke) is not loaded and
+        // adds 0; the upper pixel is loaded only where the line reaches it.
+        // lo is monotone in b, so when both pixels of the first and last band
+        // are inside the image every band's are: no checks then.
+        float x0[kBatch], x1[kBatch];
+        const int off = k * s_major;
+        if (k + 4 * (kBatch - 1) < ke && (unsigned)m0[0] < (unsigned)(n_minor - 1) &&
+            (unsigned)m0[kBatch - 1] < (unsigned)(n_minor - 1)) {
+#pragma unroll
+            for (int b = 0; b < kBatch; ++b) {
+                const int o = m0[b] * s_minor + (off + 4 * b * s_major);
+                x0[b] = ld_data<COH>(a.img + o);
+                x1[b] = c0[b] < 1.0f ? ld_data<COH>(img1 + o) : 0.0f;
+            }
+        } else {
+#pragma unroll
+            for (int b = 0; b < kBatch; ++b) {
+                const int o = m0[b] * s_minor + (off + 4 * b * s_major);
+                const bool live = k + 4 * b < ke;
+                x0[b] = live && (unsigned)m0[b] < (unsigned)n_minor ? ld_data<COH>(a.img + o) : 0.0f;
+                x1[b] = live && c0[b] < 1.0f && (unsigned)(m0[b] + 1) < (unsigned)n_minor ? ld_data<COH>(img1 + o)
+                                                                                         : 0.0f;
+            }
+        }
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b) {
+            acc = fmaf(c0[b], x0[b], acc);
+            acc = fmaf(1.0f - c0[b], x1[b], acc);
+        }
+    }
+    return acc * vp.L;
+}
+
+// The same for the consecutive bands [kb, ke), with the weights of
+// band_split() in its own rounding (states with a BF16 table, see kRefRounding).
+template <bool COH>
+__device__ __forceinline__ float walk_bands_ref(const FwdArgs &a, const ViewParams &vp, float uf, int ui, float hm,
+                                                int n_minor, int kb, int ke) {
+    const int s_major = vp.col ? 1 : a.nx;
+    const int s_minor = vp.col ? a.nx : 1;
+    const float *img1 = a.img + s_minor;
+    float acc = 0.0f;
+    float kc = (float)kb - hm;
+    float va = band_point(vp, uf, kc);
+    constexpr int kBatch = 4;
+    for (int k = kb; k < ke; k += kBatch) {
+        int m0[kBatch];
+        float c0[kBatch], c1[kBatch];
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b) {
+            kc += 1.0f;
+            const float vb = band_point(vp, uf, kc);
+            const float t = band_split_ref(vp, va, vb, c0[b], c1[b]);
+            m0[b] = (int)(__float_as_uint(t) - kRoundBits) + ui;
+            va = vb;
+        }
+        float x0[kBatch], x1[kBatch];
+        const int off = k * s_major;
+        if (k + kBatch <= ke && (unsigned)m0[0] < (unsigned)(n_minor - 1) &&
+            (unsigned)m0[kBatch - 1] < (unsigned)(n_minor - 1)) {
+#pragma unroll
+            for (int b = 0; b < kBatch; ++b) {
+                const int o = m0[b] * s_minor + (off + b * s_major);
+                x0[b] = ld_data<COH>(a.img + o);
+                x1[b] = c1[b] != 0.0f ? ld_data<COH>(img1 + o) : 0.0f;
+            }
+        } else {
+#pragma unroll
+            for (int b = 0; b < kBatch; ++b) {
+                const int o = m0[b] * s_minor + (off + b * s_major);
+                const bool live = k + b < ke;
+                x0[b] = live && (unsigned)m0[b] < (unsigned)n_minor ? ld_data<COH>(a.img + o) : 0.0f;
+                x1[b] = live && c1[b] > 0.0f && (unsigned)(m0[b] + 1) < (unsigned)n_minor ? ld_data<COH>(img1 + o)
+                                                                                         : 0.0f;
+            }
+        }
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b) {
+            acc = fmaf(c0[b], x0[b], acc);
+            acc = fmaf(c1[b], x1[b], acc);
+        }
+    }
+    return acc;
+}
+
 // Single-slice forward: a block takes RAYS adjacent rays of the view range
-// and splits each ray's bands into CHUNKS contiguous chunks (RAYS * CHUNKS =
-// kBlock).  Inside a warp, lane = 8 * chunk + ray: the 32 lanes are 8
-// adjacent rays times 4 chunks, so one warp load touches 4 image rows with
-// 8 neighbouring pixels each.  Chunk sums are reduced by xor-shuffles
-// (within the warp) and then over warps through shared memory, always in the
-// same order, so the result is deterministic.
-template <int CHUNKS, int MODE, bool LL, bool INTERIOR = true, bool COH = false, bool WIDE = false>
+// and splits each ray's bands over CHUNKS threads (RAYS * CHUNKS = kBlock): a
+// warp is 8 adjacent rays times 4 band lanes, and the CHUNKS / 4 warps of a ray
+// group take contiguous ranges of bands.  Inside a warp's range the 4 lanes
+// take every fourth band, so that one load touches 8 neighbouring pixels of 4
+// rows on a row-driven view and 4 neighbouring columns of the ~10 rows the 8
+// rays cross on a column-driven one (with contiguous chunks per lane those
+// were 32 different rows).  REF: consecutive bands per lane (kRefRounding).
+//
+// Chunk sums are reduced by xor-shuffles (within the warp) and then over
+// warps through shared memory, always in the same order, so the result is
+// deterministic.
+template <int CHUNKS, int MODE, bool LL, bool REF = false, bool COH = false, bool WIDE = false>
 __device__ __forceinline__ void forward_tile_body(const FwdArgs &a, const int bx) {
     constexpr int RAYS = kBlock / CHUNKS;        // rays per block
     constexpr int WPG = CHUNKS / 4;              // warps per group of 8 rays
@@ -43,35 +171,43 @@ __device__ __forceinline__ void forward_tile_body(const FwdArgs &a, const int bx
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const int r8 = lane & 7;
-    const int chunk = 4 * (warp % WPG) + (lane >> 3);
+    const int c4 = lane >> 3;                    // band lane
     const int ray_local = 8 * (warp / WPG) + r8;
     const int ray = bx * RAYS + ray_local;     // 32-bit: a plan has fewer than 2^31 rays
 
     // the ray's geometry: plan constants only, so it may overlap the end of
     // the kernel before this one
-    float acc = 0.0f;
     ViewParams vp{};
-    float2 u = make_float2(0.0f, 0.0f);
+    float uf = 0.0f;
     int kb = 0, ke = 0, n_minor = 0, ui = 0;
     float hm = 0.0f;
     // WIDE: a block wider than kBlock; its threads past kBlock take no ray
     if (ray < n_rays && (!WIDE || threadIdx.x < kBlock)) {
-        const int q = ray / a.nb;
+        const int q = div_by_bins(ray, a.nb_mul, a.nb_shift);
         const int j = ray - q * a.nb;
         const int v = __ldg(a.order + rr.v_begin + q);
         vp = a.views[v];
-        u = __ldg(a.uc + (long long)v * a.nb + j);
+        const float2 u = __ldg(a.uc + (long long)v * a.nb + j);
         const int n_major = vp.col ? a.nx : a.ny;
         n_minor = vp.col ? a.ny : a.nx;
         hm = 0.5f * (float)n_major;
         ui = (int)u.x + (n_minor >> 1);
+        uf = u.y;
         int k_lo, k_hi;
         band_range(vp, u.x + u.y, n_major, n_minor, k_lo, k_hi);
-        // chunks are aligned to the same bands for every ray of the view, so
-        // neighbouring lanes read the same image rows
-        const int per = (n_major + CHUNKS - 1) / CHUNKS;
-        kb = max(k_lo, chunk * per);
-        ke = min(k_hi, (chunk + 1) * per);
+        // the ranges are aligned to the same bands for every ray of the view,
+        // so neighbouring lanes read the same image rows
+        if (REF) {
+            const int per = (n_major + CHUNKS - 1) / CHUNKS;
+            const int chunk = 4 * (warp % WPG) + c4;
+            kb = max(k_lo, chunk * per);
+            ke = min(k_hi, (chunk + 1) * per);
+        } else {
+            const int per = ((n_major + WPG - 1) / WPG + 3) & ~3;
+            const int wk = (warp % WPG) * per;
+            kb = max(k_lo & ~3, wk) + c4;
+            ke = min(k_hi, wk + per);
+        }
     }
     pdl_wait();
     pdl_trigger();
@@ -86,81 +222,10 @@ __device__ __forceinline__ void forward_tile_body(const FwdArgs &a, const int bx
         if (MODE == FWD_RATIO || LL) g_f = __ldg(a.g + gi);
         if (a.w) w_f = __ldg(a.w + gi);
     }
-    {
-        if (kb < ke) {
-            const int s_major = vp.col ? 1 : a.nx;
-            const int s_minor = vp.col ? a.nx : 1;
-            float kc = (float)kb - hm;
-            float va = band_point(vp, u.y, kc);
-            // kBatch bands at a time: all their pixel offsets and weights
-            // first, then the loads, then the FMAs in band order, so that the
-            // loads of a batch are in flight together.  A piece outside the
-            // image (or of a band past ke) is not loaded and adds 0 * 0,
-            // which leaves acc unchanged: the sum is the same as with the
-            // piece skipped.
-            constexpr int kBatch = 4;
-            for (int k = kb; k < ke; k += kBatch) {
-                int o0[kBatch], o1[kBatch];
-                float c0[kBatch], c1[kBatch];
-                // Interior batch: the ray's minor position is linear in kc, so
-                // every band's pieces lie between the pixels of the batch's two
-                // end points, up to rounding that moves a floor by at most one.
-                // With one pixel of margin on each side both pieces of every
-                // band are inside the image, and the offsets need no checks
-                // (they equal the checked ones).
-                bool interior = false;
-                if (INTERIOR) {
-                    const float vend = band_point(vp, u.y, kc + (float)kBatch);
-                    const int e_lo = (int)floorf(fminf(va, vend)) + ui;
-                    const int e_hi = (int)floorf(fmaxf(va, vend)) + ui;
-                    interior = k + kBatch <= ke && e_lo >= 1 && e_hi <= n_minor - 3;
-                }
-                if (interior) {
-#pragma unroll
-                    for (int b = 0; b < kBatch; ++b) {
-                        kc += 1.0f;
-                        const float vb = band_point(vp, u.y, kc);
-                        float fl, w0, w1;
-                        band_split(vp, va, vb, fl, w0, w1);
-                        o0[b] = (k + b) * s_major + ((int)fl + ui) * s_minor;
-                        o1[b] = o0[b] + s_minor;
-                        c0[b] = w0;
-                        c1[b] = w1;
-                        va = vb;
-                    }
-                } else {
-#pragma unroll
-                    for (int b = 0; b < kBatch; ++b) {
-                        kc += 1.0f;
-                        const float vb = band_point(vp, u.y, kc);
-                        float fl, w0, w1;
-                        band_split(vp, va, vb, fl, w0, w1);
-                        const int m0 = (int)fl + ui;
-                        const bool live = k + b < ke;
-                        const bool ok0 = live && (unsigned)m0 < (unsigned)n_minor;
-                        const bool ok1 = live && w1 > 0.0f && (unsigned)(m0 + 1) < (unsigned)n_minor;
-                        const int row = (k + b) * s_major;
-                        o0[b] = ok0 ? row + m0 * s_minor : 0;
-                        o1[b] = ok1 ? row + (m0 + 1) * s_minor : 0;
-                        c0[b] = ok0 ? w0 : 0.0f;
-                        c1[b] = ok1 ? w1 : 0.0f;
-                        va = vb;
-                    }
-                }
-                float x0[kBatch], x1[kBatch];
-#pragma unroll
-                for (int b = 0; b < kBatch; ++b) {
-                    x0[b] = c0[b] != 0.0f ? ld_data<COH>(a.img + o0[b]) : 0.0f;
-                    x1[b] = c1[b] != 0.0f ? ld_data<COH>(a.img + o1[b]) : 0.0f;
-                }
-#pragma unroll
-                for (int b = 0; b < kBatch; ++b) {
-                    acc = fmaf(c0[b], x0[b], acc);
-                    acc = fmaf(c1[b], x1[b], acc);
-                }
-            }
-        }
-    }
+    float acc = 0.0f;
+    if (kb < ke)
+        acc = REF ? walk_bands_ref<COH>(a, vp, uf, ui, hm, n_minor, kb, ke)
+                  : walk_bands<COH>(a, vp, uf, ui, hm, n_minor, kb, ke);
     // the 4 chunks of each ray in this warp, then the warps of its group
     acc += __shfl_xor_sync(0xffffffffu, acc, 8);
     acc += __shfl_xor_sync(0xffffffffu, acc, 16);
@@ -208,6 +273,28 @@ __device__ __forceinline__ void forward_tile_body(const FwdArgs &a, const int bx
             a.ll_partials[bx] = s;
         }
     }
+}
+
+// One item of a batched forward, with the member's band-chunk count and rounding.
+template <int MODE, bool LL, bool COH = false, bool WIDE = false>
+__device__ __forceinline__ void forward_item(const FwdArgs &a, int shape, int bx) {
+    if constexpr (MODE == FWD_RATIO && !LL) {
+        if (a.ref) {
+            if (shape == 8)
+                forward_tile_body<8, MODE, LL, kRefRounding, COH, WIDE>(a, bx);
+            else if (shape == 16)
+                forward_tile_body<16, MODE, LL, kRefRounding, COH, WIDE>(a, bx);
+            else
+                forward_tile_body<32, MODE, LL, kRefRounding, COH, WIDE>(a, bx);
+            return;
+        }
+    }
+    if (shape == 8)
+        forward_tile_body<8, MODE, LL, false, COH, WIDE>(a, bx);
+    else if (shape == 16)
+        forward_tile_body<16, MODE, LL, false, COH, WIDE>(a, bx);
+    else
+        forward_tile_body<32, MODE, LL, false, COH, WIDE>(a, bx);
 }
 
 // Single-slice path: a block owns a kTile x kTile pixel tile.  For each view,

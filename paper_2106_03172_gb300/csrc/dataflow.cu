@@ -161,6 +161,8 @@ __global__ void __maxnreg__(kDataflowRegs)
                         a.ny = m.ny;
                         a.nz = 1;
                         a.nb = m.nb;
+                        a.nb_mul = m.nb_mul;
+                        a.nb_shift = m.nb_shift;
                         a.g = m.g;
                         a.w = m.w;
                         a.w_scalar = m.w_scalar;
@@ -169,6 +171,7 @@ __global__ void __maxnreg__(kDataflowRegs)
                         if (sg.kind == DF_FWD_UPDATE) {
                             a.sub_off = m.sub_off;
                             a.t_dev = m.seq + sg.iter;
+                            a.ref = m.ref;
                             a.out = m.ratio;
                         } else {
                             a.v_begin = 0;
@@ -242,12 +245,7 @@ __global__ void __maxnreg__(kDataflowRegs)
         if (s_ok) {
             const int kind = s_kind, shape = s_shape, bx = s_bx;
             if (kind == DF_FWD_UPDATE || kind == DF_FWD_ANCHOR) {
-                if (shape == 8)
-                    forward_tile_body<8, FWD_RATIO, false, true, true, true>(s_args.f, bx);
-                else if (shape == 16)
-                    forward_tile_body<16, FWD_RATIO, false, true, true, true>(s_args.f, bx);
-                else
-                    forward_tile_body<32, FWD_RATIO, false, true, true, true>(s_args.f, bx);
+                forward_item<FWD_RATIO, false, true, true>(s_args.f, shape, bx);
             } else if (kind == DF_FINISH) {
                 const long long i = (long long)bx * kBlock + threadIdx.x;
                 if (threadIdx.x < kBlock && i < s_args.fin.plane) finish_pixel(s_args.fin, i);

@@ -7,9 +7,8 @@
 // optionally reduces the log-likelihood sum_m g_m log yhat_m - yhat_m (§2.1,
 // Eq. (log_likelihood)) in FP64 to one partial per block.
 //
-// Thread layout: consecutive lanes share one ray, each walking a contiguous
-// chunk of the ray's major bands, then an xor-shuffle all-reduce combines
-// the chunks in a fixed order (deterministic).  Slice stacks (nz > 1) and
+// Thread layout: the band lanes of a warp share its rays (forward_tile_body),
+// then xor-shuffles combine their sums in a fixed order (deterministic).  Slice stacks (nz > 1) and
 // multi-ring lines have their own kernels in volume.cu (a warp of band chunks
 // x z-lanes per ray; the axial split of each piece).
 //
@@ -25,14 +24,13 @@ namespace petvr {
 
 namespace {
 
-// The kernels run beside the other streams' kernels: at 40 registers six
-// blocks fit on an SM (five for the full-data ratio pass, which spills at 40).
-template <int CHUNKS, bool LL>
-constexpr int fwd_min_blocks() { return CHUNKS >= 32 || LL ? 6 : 5; }
+// The kernels run beside the other streams' kernels: at 48 registers five
+// blocks fit on an SM (40 registers spill).
+constexpr int kFwdMinBlocks = 5;
 
-template <int CHUNKS, int MODE, bool LL>
-__global__ void __launch_bounds__(kBlock, fwd_min_blocks<CHUNKS, LL>()) forward_tile_kernel(const FwdArgs a) {
-    forward_tile_body<CHUNKS, MODE, LL>(a, blockIdx.x);
+template <int CHUNKS, int MODE, bool LL, bool REF = false>
+__global__ void __launch_bounds__(kBlock, kFwdMinBlocks) forward_tile_kernel(const FwdArgs a) {
+    forward_tile_body<CHUNKS, MODE, LL, REF>(a, blockIdx.x);
 }
 
 // Persistent batched forward: a resident grid whose blocks claim work items
@@ -45,7 +43,7 @@ __global__ void __launch_bounds__(kBlock, fwd_min_blocks<CHUNKS, LL>()) forward_
 // table is staged in shared memory once per block.  The body's shared arrays
 // are free again once the next claim's barrier has passed.
 template <int MODE, bool LL>
-__global__ void __launch_bounds__(kBlock, 6)
+__global__ void __launch_bounds__(kBlock, kFwdMinBlocks)
     persistent_forward_kernel(const BatchMember *ms, const WorkSeg *segs, int n_segs, int n_items, int iter,
                               int in_is_img, int *claim) {
     __shared__ WorkSeg s_segs[kSegSmem];
@@ -76,6 +74,8 @@ __global__ void __launch_bounds__(kBlock, 6)
                 a.ny = m.ny;
                 a.nz = 1;
                 a.nb = m.nb;
+                a.nb_mul = m.nb_mul;
+                a.nb_shift = m.nb_shift;
                 a.g = m.g;
                 a.w = m.w;
                 a.w_scalar = m.w_scalar;
@@ -83,6 +83,7 @@ __global__ void __launch_bounds__(kBlock, 6)
                 if (sg.kind == WK_FWD_UPDATE) {
                     a.sub_off = m.sub_off;
                     a.t_dev = m.seq + iter;
+                    a.ref = m.ref;
                     a.img = in_is_img ? m.img : m.alt;
                     a.out = m.ratio;
                 } else if (sg.kind == WK_FWD_ANCHOR) {
@@ -103,13 +104,7 @@ __global__ void __launch_bounds__(kBlock, 6)
         }
         __syncthreads();
         if (s_item >= n_items) break;
-        const int bx = s_bx;
-        if (s_shape == 8)
-            forward_tile_body<8, MODE, LL>(s_a, bx);
-        else if (s_shape == 16)
-            forward_tile_body<16, MODE, LL>(s_a, bx);
-        else
-            forward_tile_body<32, MODE, LL>(s_a, bx);
+        forward_item<MODE, LL>(s_a, s_shape, s_bx);
     }
 }
 
@@ -156,7 +151,9 @@ __global__ void __launch_bounds__(kBlock) count_nnz_kernel(const FwdArgs a, unsi
 template <int CHUNKS>
 pet_status dispatch_tile(const FwdArgs &a, int mode, bool ll, int blocks, cudaStream_t s) {
     void (*k)(FwdArgs) = nullptr;
-    if (mode == FWD_YHAT && !ll)
+    if (a.ref && mode == FWD_RATIO && !ll)
+        k = forward_tile_kernel<CHUNKS, FWD_RATIO, false, kRefRounding>;
+    else if (mode == FWD_YHAT && !ll)
         k = forward_tile_kernel<CHUNKS, FWD_YHAT, false>;
     else if (mode == FWD_RATIO && !ll)
         k = forward_tile_kernel<CHUNKS, FWD_RATIO, false>;

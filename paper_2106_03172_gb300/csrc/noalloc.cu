@@ -88,6 +88,8 @@ extern "C" pet_status pet_objective_noalloc(const pet_plan *plan, const float *d
     a.ny = plan->ny;
     a.nz = plan->nz;
     a.nb = plan->nb;
+    a.nb_mul = plan->nb_mul;
+    a.nb_shift = plan->nb_shift;
     a.img = d_img;
     a.g = d_counts;
     a.w = d_bg;

@@ -44,7 +44,7 @@ namespace petvr {
 // value and its FP64 rounding residual), and u - ui is evaluated as
 // uf + kc (du + du_lo), whose magnitude stays small exactly when |du| is.
 // ---------------------------------------------------------------------------
-struct ViewParams {
+struct alignas(16) ViewParams {
     float du;     // minor displacement (pixels) per major step (FP32 value)
     float du_lo;  // FP64 residual du_exact - du
     float L;      // ray length (mm) per major step
@@ -54,7 +54,21 @@ struct ViewParams {
     float inv_du; // 1 / du (0 if du == 0), for band ranges only
     float uc0;    // centred minor coordinate of bin 0 at the central major line (approx.)
     int col;      // 1: major axis is x (columns); 0: major axis is y (rows)
+    float inv_adu; // 1 / |du| (kAxisInv if du == 0), for the piece shares
+    float pad[2];
 };
+
+// inv_adu of an axis-aligned view: a share saturates to 0 or 1 for any offset
+// from a pixel edge above 1 / kAxisInv, and products with it stay finite.
+constexpr float kAxisInv = 1e30f;
+
+// Adding kRound to a float of magnitude below 2^22 leaves its integer part in
+// the low mantissa bits, rounded the way the addition rounds: the integer as
+// a float is (x + kRound) - kRound, and as an int the bit pattern minus
+// kRoundBits.  Both conversions run at the full FP32/integer rate, where
+// floorf and the float-to-int conversion run at a quarter of it.
+constexpr float kRound = 12582912.0f;          // 1.5 * 2^23
+constexpr unsigned kRoundBits = 0x4B400000u;
 
 // Bands [k_lo, k_hi) where a ray with centred minor offset uc can meet the
 // image (a superset with one band of margin each side; extra bands add 0).
@@ -99,6 +113,27 @@ __device__ __forceinline__ void band_split(const ViewParams &vp, float va, float
         w0 = fminf((fl + 1.0f - lo) * vp.Lm, vp.L);
         w1 = vp.L - w0;
     }
+}
+
+// band_split() with the floor by a directed-rounding add: the same weights,
+// bit for bit (the results of comparisons and roundings do not change), and
+// kRound + floor(lo) in place of the floor.
+__device__ __forceinline__ float band_split_ref(const ViewParams &vp, float va, float vb, float &w0, float &w1) {
+    const float lo = fminf(va, vb);
+    const float t = __fadd_rd(lo, kRound);
+    const float fl1 = t - (kRound - 1.0f);
+    const float part = fminf((fl1 - lo) * vp.Lm, vp.L);
+    w0 = fmaxf(va, vb) <= fl1 ? vp.L : part;
+    w1 = vp.L - w0;
+    return t;
+}
+
+// Share of a band (as a fraction of its length) in the lower of the two minor
+// pixels it can touch, for the band's lower end `lo` and fl1 = floor(lo) + 1:
+// the line covers inv_adu of a band per pixel of minor displacement, so the
+// lower pixel gets min((fl1 - lo) / |du|, 1) and the upper one the rest.
+__device__ __forceinline__ float band_share(float fl1, float lo, float inv_adu) {
+    return __saturatef((fl1 - lo) * inv_adu);
 }
 
 // ---------------------------------------------------------------------------
@@ -224,6 +259,15 @@ cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, s
 // ---------------------------------------------------------------------------
 // Kernel argument blocks.
 // ---------------------------------------------------------------------------
+// Which rounding a single-slice projection takes.  A BF16 table keeps 8 bits
+// of each subset gradient, so an ulp in a projection moves the entries that lie
+// on a rounding boundary by 2^-8 of themselves (measured: 2.5e-5 of an image
+// after three updates, where FP32 states stay within 1e-6).  States with such
+// a table, and the sensitivities their entries subtract, therefore keep the
+// rounding of band_split() and the order of its sums bit for bit; all others
+// take the cheaper band_share() form, which is as close to the exact weights.
+constexpr bool kRefRounding = true;
+
 enum FwdMode { FWD_NONE = 0, FWD_YHAT = 1, FWD_RATIO = 2 };
 
 struct FwdArgs {
@@ -235,6 +279,8 @@ struct FwdArgs {
     const int *sub_off;       //   [sub_off[t], sub_off[t+1]) and g / w are the full
                               //   subset-major arrays (offset applied on the device)
     int nx, ny, nz, nb;       // nz: entries per (view, bin): slices, or ring pairs (lz set)
+    unsigned nb_mul;          // division of a ray index by nb (div_by_bins)
+    int nb_shift;
     int layers;               // multi-ring: image layers (voxel index = pixel * layers + iz)
     const float4 *lz;         // multi-ring: axial table per line, [view][bin][pair]; else null
     const float *img;         // [ny][nx][nz] ([ny][nx][layers] multi-ring)
@@ -244,11 +290,23 @@ struct FwdArgs {
     float *out;               // compact output (yhat or ratio)
     double *ll_partials;      // per-block partial log-likelihood (LL only)
     int *status;              // device error latch (may be null)
+    int ref;                  // single slices: kRefRounding
 };
 
 // View range of a forward launch: given on the host, or (t_dev set) read on
 // the device from the subset offsets, with the element offset of the range's
 // first ray into the subset-major counts / background.
+// n / nb for 0 <= n < 2^31, by multiplication: with s = ceil(log2 nb) and
+// mul = ceil(2^(31 + s) / nb) < 2^32 (bins_division), (n mul) >> (31 + s) is exact.
+inline void bins_division(int nb, unsigned &mul, int &shift) {
+    shift = 0;
+    while ((1LL << shift) < nb) ++shift;
+    mul = (unsigned)(((1ULL << (31 + shift)) + (unsigned)nb - 1) / (unsigned)nb);
+}
+__device__ __forceinline__ int div_by_bins(int n, unsigned mul, int shift) {
+    return (int)(__umulhi(2u * (unsigned)n, mul) >> shift);
+}
+
 struct RayRange {
     int v_begin, v_end;
     long long off;   // element offset of the range's first ray in g / w (compact layouts)
@@ -339,6 +397,8 @@ struct BatchMember {
     const int *order;
     const int *sub_off;
     int nx, ny, nb, ns;
+    unsigned nb_mul;       // division by nb (FwdArgs)
+    int nb_shift;
     const float *sens_t;
     const float *sens;
     const float *g;
@@ -349,6 +409,7 @@ struct BatchMember {
     float delta;
     int *status;
     int algo, table_dtype;
+    int ref;               // kRefRounding
     float *img, *alt, *ratio;
     float *ratio_full;     // anchor-pass ratio over all views (SVREM, SVRG), subset-major
     float *s_hat;
@@ -453,6 +514,8 @@ struct pet_plan {
     int device;
     int fwd_chunks = 0;             // single-slice forward: band chunks per ray (8, 16 or 32)
     int back_run = 8;               // single-slice back projection: pixels per run (4 or 8)
+    unsigned nb_mul = 0;            // division of a ray index by nb (bins_division)
+    int nb_shift = 0;
     std::vector<int> order;         // subset-major view order
     std::vector<int> sub_off;       // [ns + 1]
     std::vector<long long> nnz;     // [ns] nonzeros of A_t (one slice)
@@ -487,6 +550,7 @@ struct pet_batch;
 struct pet_state {
     const pet_problem *prob;
     int algo, table_dtype;
+    int ref;               // kRefRounding
     float *img;                     // caller's image (current iterate)
     float *alt = nullptr;           // ping-pong partner
     float *ratio = nullptr;         // [max subset rays * nz]
