@@ -163,7 +163,9 @@ BackArgs back_args(const pet_plan *pl, const float *r, int subset, bool natural)
     a.r = r;
     a.sens_t = pl->d_sens_t;
     a.sens = pl->d_sens;
-    a.run = pl->back_run;
+    a.bw = pl->bw;
+    a.cand1 = pl->cand1;
+    a.cand2 = pl->cand2;
     return a;
 }
 
@@ -184,7 +186,42 @@ pet_status ratio_subset(const pet_problem *p, const float *f, int t, float *rati
 
 // Whether a state's projections keep the reference rounding (kRefRounding).
 int ref_rounding(const pet_state *st) {
-    return st->algo == PET_ALGO_SAGA && st->table_dtype == PET_TABLE_BF16 ? 1 : 0;
+    const pet_plan *pl = st->prob->plan;
+    return st->algo == PET_ALGO_SAGA && st->table_dtype == PET_TABLE_BF16 && pl->nz == 1 && !pl->ring ? 1 : 0;
+}
+
+// Sensitivities of the reference rounding, of every subset and their sum (a
+// state's gradient subtracts the sensitivity of its own projector: other
+// rounding there would not cancel).  Made when the first state that needs them is, and kept by the plan.
+pet_status ensure_ref_sensitivity(const pet_plan *pl, cudaStream_t s) {
+    std::lock_guard<std::mutex> lk(pl->ref_mu);
+    if (pl->d_sens_t_ref) return PET_OK;
+    float *ones = nullptr, *sens = nullptr;
+    pet_status st = dalloc(&ones, (size_t)pl->M, "ones");
+    if (st == PET_OK) st = dalloc(&sens, (size_t)(pl->ns + 1) * pl->N, "reference sensitivities");
+    if (st == PET_OK) {
+        const std::vector<float> h1((size_t)pl->M, 1.0f);
+        st = cuda_ok(cudaMemcpyAsync(ones, h1.data(), sizeof(float) * pl->M, cudaMemcpyHostToDevice, s), "ones upload");
+        if (st == PET_OK) {
+            BackArgs b = back_args(pl, ones, -1, false);
+            b.t0 = 0;
+            b.r_view0 = 0;
+            b.out = sens;
+            b.ref = 1;
+            st = launch_back(b, EPI_ANCHOR, PET_TABLE_FP32, pl->ns, s, pl->max_sub_views);
+            if (st == PET_OK) st = launch_sum_sens(sens, sens + (size_t)pl->ns * pl->N, pl->ns, pl->N, s);
+        }
+        // other streams' states read them next, and `ones` is freed
+        const pet_status done = cuda_ok(cudaStreamSynchronize(s), "reference sensitivities");
+        if (st == PET_OK) st = done;
+    }
+    dfree(ones);
+    if (st != PET_OK) {
+        dfree(sens);
+        return st;
+    }
+    pl->d_sens_t_ref = sens;
+    return PET_OK;
 }
 
 // Full-data ratio in subset-major order into `ratio` (M * nz).
@@ -287,9 +324,10 @@ pet_status state_init(pet_state *st, cudaStream_t s) {
     b.pot = p->pen.potential;
     b.delta = p->pen.delta;
     b.table = st->table;
+    if (ref_rounding(st)) b.sens_t = pl->d_sens_t_ref;
     PET_TRY(launch_back(b, EPI_SAGA_INIT, st->table_dtype, pl->ns, s, pl->max_sub_views));
-    return launch_saga_finish(st->table, st->table_dtype, pl->ns, Nz, pl->nz, st->img, pl->d_sens, st->qbar, st->d,
-                              s);
+    const float *sens = ref_rounding(st) ? pl->d_sens_t_ref + (size_t)pl->ns * pl->N : pl->d_sens;
+    return launch_saga_finish(st->table, st->table_dtype, pl->ns, Nz, pl->nz, st->img, sens, st->qbar, st->d, s);
 }
 
 // The warm start (a constant image, then one unpenalised OSEM epoch in cyclic
@@ -383,6 +421,7 @@ void pet_plan_destroy(pet_plan *pl) {
     dfree(pl->d_all_off);
     dfree(pl->d_sens_t);
     dfree(pl->d_sens);
+    dfree(pl->d_sens_t_ref);
     dfree(pl->d_lz);
     delete pl;
 }
@@ -427,6 +466,7 @@ pet_status pet_plan_create(const pet_geometry *g, const pet_subsets *sub, pet_pl
     pl->na = g->n_angles;
     pl->nb = g->n_bins;
     bins_division(pl->nb, pl->nb_mul, pl->nb_shift);
+    tile_bins(g->pixel_mm, ds_chk, pl->nb, pl->nx, pl->ny, pl->bw, pl->cand1, pl->cand2);
     pl->ns = sub->n_subsets;
     pl->N = (int)N;
     pl->M = (int)M;
@@ -533,6 +573,7 @@ pet_status pet_plan_create(const pet_geometry *g, const pet_subsets *sub, pet_pl
     b.t0 = 0;
     b.r_view0 = 0;
     b.out = pl->d_sens_t;
+    b.ref = !ring && g->nz > 1 ? 1 : 0;
     if ((st = launch_back(b, EPI_ANCHOR, PET_TABLE_FP32, pl->ns, 0, pl->max_sub_views)) != PET_OK) return fail(st);
     if ((st = launch_sum_sens(pl->d_sens_t, pl->d_sens, pl->ns, pl->N, 0)) != PET_OK) return fail(st);
     // nonzeros per subset, counted with the projector's own geometry
@@ -581,6 +622,8 @@ pet_status pet_plan_bytes(const pet_plan *pl, size_t *h_bytes) {
     if (!pl || !h_bytes) return set_error(PET_ERR_INVALID, "null argument");
     *h_bytes = sizeof(ViewParams) * pl->na + sizeof(float2) * (size_t)pl->M + sizeof(int) * (2 * (size_t)pl->na + pl->ns + 3) +
                sizeof(float) * ((size_t)pl->ns + 1) * pl->N;
+    std::lock_guard<std::mutex> lk(pl->ref_mu);
+    if (pl->d_sens_t_ref) *h_bytes += sizeof(float) * ((size_t)pl->ns + 1) * pl->N;
     return PET_OK;
 }
 
@@ -620,26 +663,23 @@ pet_status pet_plan_autotune(pet_plan *pl, int32_t *h_fwd_chunks, int32_t *h_bac
     if (!pl) return set_error(PET_ERR_INVALID, "null plan");
     if (pl->nz == 1 && !pl->ring) {
         const size_t N = (size_t)pl->N, R = (size_t)max_sub_rays(pl);
-        float *img = nullptr, *sino = nullptr, *out = nullptr;
+        float *img = nullptr, *sino = nullptr;
         cudaStream_t s = nullptr;
         cudaEvent_t e0 = nullptr, e1 = nullptr;
         pet_status st = PET_OK;
         auto cleanup = [&]() {
             dfree(img);
             dfree(sino);
-            dfree(out);
             if (e0) cudaEventDestroy(e0);
             if (e1) cudaEventDestroy(e1);
             if (s) cudaStreamDestroy(s);
         };
-        if ((st = dalloc(&img, N, "tune image")) != PET_OK || (st = dalloc(&sino, R, "tune sinogram")) != PET_OK ||
-            (st = dalloc(&out, N, "tune image")) != PET_OK) {
+        if ((st = dalloc(&img, N, "tune image")) != PET_OK || (st = dalloc(&sino, R, "tune sinogram")) != PET_OK) {
             cleanup();
             return st;
         }
-        std::vector<float> ones(std::max(N, R), 1.0f);
+        std::vector<float> ones(N, 1.0f);
         cudaError_t e = cudaMemcpy(img, ones.data(), N * 4, cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy(sino, ones.data(), R * 4, cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaEventCreate(&e0);
         if (e == cudaSuccess) e = cudaEventCreate(&e1);
@@ -647,21 +687,15 @@ pet_status pet_plan_autotune(pet_plan *pl, int32_t *h_fwd_chunks, int32_t *h_bac
             cleanup();
             return cuda_ok(e, "autotune set-up");
         }
-        // time `reps` passes over every subset of one projector, best of 3
-        auto time_pass = [&](bool forward, float *best_ms) -> pet_status {
+        // time passes over every subset's forward projection, best of 3
+        auto time_pass = [&](float *best_ms) -> pet_status {
             float best = 1e30f;
             for (int trial = 0; trial < 4; ++trial) {
                 PET_TRY(cuda_ok(cudaEventRecord(e0, s), "event"));
                 for (int t = 0; t < pl->ns; ++t) {
-                    if (forward) {
-                        FwdArgs a = fwd_args(pl, img, t, false);
-                        a.out = sino;
-                        PET_TRY(launch_forward(a, FWD_YHAT, false, choose_group(pl), s, nullptr));
-                    } else {
-                        BackArgs b = back_args(pl, sino, t, false);
-                        b.out = out;
-                        PET_TRY(launch_back(b, EPI_PLAIN, PET_TABLE_FP32, 1, s, pl->max_sub_views));
-                    }
+                    FwdArgs a = fwd_args(pl, img, t, false);
+                    a.out = sino;
+                    PET_TRY(launch_forward(a, FWD_YHAT, false, choose_group(pl), s, nullptr));
                 }
                 PET_TRY(cuda_ok(cudaEventRecord(e1, s), "event"));
                 PET_TRY(cuda_ok(cudaEventSynchronize(e1), "event sync"));
@@ -672,30 +706,15 @@ pet_status pet_plan_autotune(pet_plan *pl, int32_t *h_fwd_chunks, int32_t *h_bac
             *best_ms = best;
             return PET_OK;
         };
-        int best_c = choose_group(pl), best_r = pl->back_run;
+        int best_c = choose_group(pl);
         float best_ms = 1e30f;
         for (int c : {8, 16, 32}) {
             pl->fwd_chunks = c;
             float ms = 0.0f;
-            if ((st = time_pass(true, &ms)) != PET_OK) break;
+            if ((st = time_pass(&ms)) != PET_OK) break;
             if (ms < best_ms) best_ms = ms, best_c = c;
         }
         pl->fwd_chunks = best_c;
-        best_ms = 1e30f;
-        // 4-pixel runs need blocks twice as wide as 8-pixel runs, so fewer fit
-        // beside other streams' kernels and the all-subset launches (anchors,
-        // table fills) slow down: measured on the 256^2 four-stream step, run 4
-        // took its subset back projections from 9.6 to 10.4 us and its anchor
-        // from 47 to 93 us, and the step from 28.2 to 40.6 ms.  Timed alone the
-        // two are close, so run 4 is taken only when it is clearly faster.
-        for (int r : {8, 4}) {
-            if (st != PET_OK) break;
-            pl->back_run = r;
-            float ms = 0.0f;
-            if ((st = time_pass(false, &ms)) != PET_OK) break;
-            if (ms < best_ms * (r == 4 ? 0.85f : 1.0f)) best_ms = ms, best_r = r;
-        }
-        pl->back_run = best_r;
         cleanup();
         if (st != PET_OK) return st;
     }
@@ -909,6 +928,7 @@ pet_status pet_state_create(const pet_problem *p, int32_t algo, int32_t table_dt
             return fail(set_error(PET_ERR_OOM, "cudaMalloc SAGA table"));
         }
     }
+    if (ref_rounding(st) && (e = ensure_ref_sensitivity(pl, s)) != PET_OK) return fail(e);
     if ((e = state_init(st, s)) != PET_OK) return fail(e);
     *out = st;
     return PET_OK;
@@ -965,6 +985,7 @@ pet_status enqueue_update(pet_state *st, int algo, const int *t_dev, const float
         b.B = st->B;
     } else if (algo == PET_ALGO_SAGA) {
         epi = EPI_SAGA;
+        if (ref_rounding(st)) b.sens_t = pl->d_sens_t_ref;
         b.d = st->precond == PET_PRECOND_ITERATE ? nullptr : st->d;
         b.table = st->table;
         b.qbar = st->qbar;
@@ -1840,8 +1861,11 @@ void fill_member(BatchMember &m, const pet_state *st, float alpha, const int *se
     m.nb = pl->nb;
     m.nb_mul = pl->nb_mul;
     m.nb_shift = pl->nb_shift;
+    m.bw = pl->bw;
+    m.cand1 = pl->cand1;
+    m.cand2 = pl->cand2;
     m.ns = pl->ns;
-    m.sens_t = pl->d_sens_t;
+    m.sens_t = ref_rounding(st) ? pl->d_sens_t_ref : pl->d_sens_t;
     m.sens = pl->d_sens;
     m.g = p->d_g;
     m.w = p->d_w;
@@ -1882,8 +1906,9 @@ void fill_member(BatchMember &m, const pet_state *st, float alpha, const int *se
 //     the other members' updates, the anchor finishes, then a back phase with
 //     the anchored members' updates; otherwise one back phase with every
 //     member's update.
-// Back phases are split by potential class (the quadratic epilogue and the
-// edge-preserving one are different kernels), longest tiles first.
+// Back phases are split by potential class and rounding (the quadratic epilogue
+// and the edge-preserving one, and the reference rounding of BF16 tables, are
+// different kernels), longest tiles first.
 // PET_BATCH_STREAMS: the batch's own streams (up to 8), created on first use;
 // fork makes them wait for `s`, join makes `s` wait for them.
 constexpr int kBatchSideStreams = 8;
@@ -1921,15 +1946,12 @@ void build_batch_phases(pet_batch *b, int n_iter, const std::vector<std::vector<
     int claim = 0;
     auto tiles_of = [](const pet_plan *pl) { return ((pl->nx + 15) / 16) * ((pl->ny + 15) / 16); };
     auto major_of = [](const pet_plan *pl) { return std::max(pl->nx, pl->ny); };
-    auto emit = [&](int i, int kind, std::vector<WorkSeg> &segs, int genpot) {
+    auto emit = [&](int i, int kind, std::vector<WorkSeg> &segs, int genpot, int ref) {
         if (segs.empty()) return;
-        pet_batch::Phase ph{kind, (int)b->h_segs.size(), (int)segs.size(), 0, 256, genpot, claim++};
+        pet_batch::Phase ph{kind, (int)b->h_segs.size(), (int)segs.size(), 0, genpot, ref, claim++};
         for (WorkSeg &g : segs) {
             g.first = ph.n_items;
             ph.n_items += g.count;
-            if (kind == 1)
-                ph.threads = std::max(ph.threads, back_block_threads(g.shape,
-                                                                     b->states[g.member]->prob->plan->max_sub_views));
             b->h_segs.push_back(g);
         }
         b->phases[(size_t)i].push_back(ph);
@@ -1955,28 +1977,29 @@ void build_batch_phases(pet_batch *b, int n_iter, const std::vector<std::vector<
         std::stable_sort(fa.begin(), fa.end(), longer_fwd);
         std::stable_sort(fu.begin(), fu.end(), longer_fwd);
         fa.insert(fa.end(), fu.begin(), fu.end());
-        emit(i, 0, fa, 0);
+        emit(i, 0, fa, 0, 0);
         // views per subset decide a back item's length
         auto longer_back = [&](const WorkSeg &x, const WorkSeg &y) {
             return b->states[x.member]->prob->plan->max_sub_views > b->states[y.member]->prob->plan->max_sub_views;
         };
         for (int pass = any ? 0 : 1; pass < 2; ++pass) {
-            for (int gp = 0; gp < 2; ++gp) {
+            for (int cls = 0; cls < 4; ++cls) {
+                const int gp = cls & 1, ref = cls >> 1;
                 std::vector<WorkSeg> anc, upd;
                 for (int j = 0; j < n; ++j) {
                     const pet_state *st = b->states[j];
                     const pet_plan *pl = st->prob->plan;
                     const int member_gp = st->prob->pen.potential != PET_POT_QUADRATIC ? 1 : 0;
-                    if (pass == 0 && anchors[j][i] && gp == 0)
-                        anc.push_back({j, WK_BACK_ANCHOR, 0, tiles_of(pl) * pl->ns, pl->back_run, tiles_of(pl)});
+                    if (pass == 0 && anchors[j][i] && cls == 0)
+                        anc.push_back({j, WK_BACK_ANCHOR, 0, tiles_of(pl) * pl->ns, 0, tiles_of(pl)});
                     const bool update_here = any ? ((pass == 0) != (anchors[j][i] != 0)) : true;
-                    if (update_here && member_gp == gp)
-                        upd.push_back({j, WK_BACK_UPDATE, 0, tiles_of(pl), pl->back_run, tiles_of(pl)});
+                    if (update_here && member_gp == gp && ref_rounding(st) == ref)
+                        upd.push_back({j, WK_BACK_UPDATE, 0, tiles_of(pl), 0, tiles_of(pl)});
                 }
                 std::stable_sort(anc.begin(), anc.end(), longer_back);
                 std::stable_sort(upd.begin(), upd.end(), longer_back);
                 anc.insert(anc.end(), upd.begin(), upd.end());
-                emit(i, 1, anc, gp);
+                emit(i, 1, anc, gp, ref);
             }
             if (pass == 0) b->phases[(size_t)i].push_back({2, 0, 0, 0, 0, 0, -1});   // the anchor finishes
         }
@@ -1987,22 +2010,20 @@ void build_batch_phases(pet_batch *b, int n_iter, const std::vector<std::vector<
 // The dependency-driven epoch's work list (into b->h_df): every stage of every
 // member, merged stage by stage across members (each member's k-th stage
 // before any member's (k+1)-th), with each stage's needs (see dataflow.cu).
-// Returns the block size and whether the members use an edge-preserving
-// potential (all must share one potential class).
-int build_batch_dataflow(pet_batch *b, int n_iter, const std::vector<std::vector<uint8_t>> &anchors, bool *genpot) {
+// Also tells whether the members use an edge-preserving potential (all must
+// share one potential class).
+void build_batch_dataflow(pet_batch *b, int n_iter, const std::vector<std::vector<uint8_t>> &anchors, bool *genpot) {
     const int n = (int)b->states.size();
     struct Stage {
         DfSeg seg;
         int dep0, dep1;   // indices into the member's own stage list (-1: none)
     };
     std::vector<std::vector<Stage>> lists((size_t)n);
-    int threads = 256;
     *genpot = b->states[0]->prob->pen.potential != PET_POT_QUADRATIC;
     for (int j = 0; j < n; ++j) {
         const pet_state *st = b->states[j];
         const pet_plan *pl = st->prob->plan;
         const int tiles = ((pl->nx + 15) / 16) * ((pl->ny + 15) / 16);
-        threads = std::max(threads, back_block_threads(pl->back_run, pl->max_sub_views));
         bool ready = st->s_hat_ready;
         int prev_b = -1;
         auto add = [&](int kind, int count, int shape, int iter, int flag, int d0, int d1) {
@@ -2015,14 +2036,14 @@ int build_batch_dataflow(pet_batch *b, int n_iter, const std::vector<std::vector
             if (anchors[j][i]) {
                 const int af = add(DF_FWD_ANCHOR, forward_blocks(pl->M, 1, full_group(pl)), full_group(pl), i, 0,
                                    prev_b, -1);
-                const int ab = add(DF_BACK_ANCHOR, tiles * pl->ns, pl->back_run, i, 0, af, -1);
+                const int ab = add(DF_BACK_ANCHOR, tiles * pl->ns, 0, i, 0, af, -1);
                 fin = add(DF_FINISH, (int)((plane_of(pl) + 255) / 256), 0, i,
                           st->algo == PET_ALGO_SVREM && !ready ? 1 : 0, ab, -1);
                 if (st->algo == PET_ALGO_SVREM) ready = true;
             }
             const int f = add(DF_FWD_UPDATE, forward_blocks(max_sub_rays(pl), 1, choose_group(pl)),
                               choose_group(pl), i, 0, prev_b, -1);
-            prev_b = add(DF_BACK_UPDATE, tiles, pl->back_run, i, 0, f, fin);
+            prev_b = add(DF_BACK_UPDATE, tiles, 0, i, 0, f, fin);
         }
     }
     // merge stage by stage; map each member's stage indices to list positions
@@ -2049,12 +2070,11 @@ int build_batch_dataflow(pet_batch *b, int n_iter, const std::vector<std::vector
             pos[(size_t)j][k] = (int)b->h_df.size();
             b->h_df.push_back(stg.seg);
         }
-    return threads;
 }
 
 // The dependency-driven epoch on stream s: the iterate copy (odd update
 // counts), SEM statistics due, the counters' reset, then one launch.
-pet_status enqueue_batch_dataflow(pet_batch *b, int32_t n_iter, int threads, bool genpot, cudaStream_t s) {
+pet_status enqueue_batch_dataflow(pet_batch *b, int32_t n_iter, bool genpot, cudaStream_t s) {
     const bool odd = (n_iter % 2) == 1;
     if (odd)
         for (pet_state *st : b->states) {
@@ -2071,7 +2091,7 @@ pet_status enqueue_batch_dataflow(pet_batch *b, int32_t n_iter, int threads, boo
     const DfSeg &last = b->h_df.back();
     PET_TRY(launch_zero_ints(b->d_df_done, n_segs + 1, s));
     return launch_dataflow_epoch(b->d_members, b->d_df, n_segs, last.first + last.count, odd ? 1 : 0, b->d_df_done,
-                                 b->d_status, b->wait_limit, genpot, threads, s);
+                                 b->d_status, b->wait_limit, genpot, s);
 }
 
 // All launches of one batched epoch on stream s (phases from build_batch_phases).
@@ -2101,8 +2121,7 @@ pet_status enqueue_batch_epoch(pet_batch *b, int32_t n_iter, const std::vector<s
                                                   in_is_img ? 1 : 0, b->d_claims + ph.claim, false, s));
             } else if (ph.kind == 1) {
                 PET_TRY(launch_persistent_back(b->d_members, b->d_segs + ph.seg_off, ph.n_segs, ph.n_items, i,
-                                               in_is_img ? 1 : 0, b->d_claims + ph.claim, ph.genpot != 0, ph.threads,
-                                               s));
+                                               in_is_img ? 1 : 0, b->d_claims + ph.claim, ph.genpot != 0, ph.ref != 0, s));
             } else {
                 for (int j = 0; j < n; ++j) {
                     if (!anchors[j][i]) continue;
@@ -2206,7 +2225,7 @@ pet_status pet_batch_epoch(pet_batch *b, const int32_t *h_seqs, int32_t n_iter, 
                              (b->states[0]->prob->pen.potential != PET_POT_QUADRATIC);
     if (b->mode == PET_BATCH_DATAFLOW && uniform_potential) {
         bool genpot = false;
-        const int threads = build_batch_dataflow(b, n_iter, anchors, &genpot);
+        build_batch_dataflow(b, n_iter, anchors, &genpot);
         const int n_segs = (int)b->h_df.size();
         if (n_segs > b->df_cap || n_segs + 1 > b->df_done_cap) {
             DfSeg *grown = nullptr;
@@ -2233,14 +2252,14 @@ pet_status pet_batch_epoch(pet_batch *b, const int32_t *h_seqs, int32_t n_iter, 
         pet_status rc;
         key.push_back(-1);   // this mode's graphs apart from the phases'
         if (direct) {
-            rc = enqueue_batch_dataflow(b, n_iter, threads, genpot, s);
+            rc = enqueue_batch_dataflow(b, n_iter, genpot, s);
         } else {
             pet_state holder{};
             holder.cap = b->cap;
             holder.graphs.swap(b->graphs);
             holder.graph_tick = b->graph_tick;
             rc = run_graph(&holder, key, s,
-                           [&](cudaStream_t cs) { return enqueue_batch_dataflow(b, n_iter, threads, genpot, cs); });
+                           [&](cudaStream_t cs) { return enqueue_batch_dataflow(b, n_iter, genpot, cs); });
             b->graphs.swap(holder.graphs);
             b->graph_tick = holder.graph_tick;
             b->cap = holder.cap;

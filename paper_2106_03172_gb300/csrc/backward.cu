@@ -2,8 +2,8 @@
 // update of each method (K3).
 //
 // b_n = sum_{m in S_t} a_mn r_m as a gather per pixel (no atomics, so the
-// result is deterministic).  Single slices use tiles with runs of pixels
-// that share each ray's band split (back_tile_kernel, here); slice stacks
+// result is deterministic).  Single slices use tiles that stage the bins they
+// need of every view (back_tile_kernel, here); slice stacks
 // and multi-ring volumes have their own kernels in volume_back.cu (z-lanes
 // over a pixel's slices; each band piece split over the layers its axial
 // range crosses).  In each view only the bins whose ray
@@ -26,6 +26,7 @@
 //   ANCHOR B_t = b for every subset t at once (grid.y = t)
 //   SAGA_INIT table_t = b - sens_t - (beta/N_s) grad R(f) for every t.
 #include <algorithm>
+#include <type_traits>
 
 #include "bodies.cuh"
 
@@ -33,64 +34,42 @@ namespace petvr {
 
 namespace {
 
-// The all-subset launches (anchor passes, table fills), the full-data
-// statistic and plain back projections run in back_tile_wide_kernel, capped at
-// 48 registers: four 288-thread blocks per SM where the compiler's own choice
-// (57) leaves three.  The subset updates keep theirs (42).
-constexpr bool wide_epilogue(int epi) {
-    return epi == EPI_ANCHOR || epi == EPI_SAGA_INIT || epi == EPI_SAGAEM_INIT || epi == EPI_SEM_INIT ||
-           epi == EPI_PLAIN;
-}
-constexpr int kWideRegs = 48;
-static_assert(kTile * kTile == kBlock, "one pixel of the tile per thread");
+// Pixels a thread of the tile kernels takes (blocks of kTile^2 / PX threads per
+// group): two on launches over several subsets and in the persistent batches.
+constexpr int kPx = 2;
+constexpr int tile_threads(int px) { return kTile * kTile / px; }
+// Launches over this many views at once (all-view back projections, the SEM
+// start) split them over kViewGroups groups of threads per tile.
+constexpr int kManyViews = 32;
 
-template <int EPI, typename TQ, int kRun, bool GENPOT>
-__global__ void __launch_bounds__(kTileBlockMax) back_tile_kernel(const BackArgs a) {
+template <int EPI, typename TQ, bool GENPOT, int PX, int GROUPS = 1>
+__global__ void __launch_bounds__(tile_threads(PX) * GROUPS, 4 * PX / GROUPS) back_tile_kernel(const BackArgs a) {
     const int t = a.t_dev ? __ldg(a.t_dev) : a.t0 + (int)blockIdx.y;
-    back_tile_body<EPI, TQ, kRun, GENPOT>(a, t, blockIdx.x);
+    back_tile_body<EPI, TQ, GENPOT, PX, false, GROUPS>(a, t, blockIdx.x);
 }
 
-template <int EPI, typename TQ, int kRun, bool GENPOT>
-__global__ void __maxnreg__(kWideRegs) back_tile_wide_kernel(const BackArgs a) {
+template <int EPI, typename TQ, bool GENPOT>
+__global__ void __launch_bounds__(kRunThreadsMax) back_run_kernel(const BackArgs a) {
     const int t = a.t_dev ? __ldg(a.t_dev) : a.t0 + (int)blockIdx.y;
-    back_tile_body<EPI, TQ, kRun, GENPOT>(a, t, blockIdx.x);
-}
-
-// Member update of one tile: the member's algorithm and table type select
-// the epilogue (the single-state launch's template arguments).
-template <int kRun, bool GENPOT>
-__device__ __forceinline__ void member_update_tile(int algo, int table_dtype, const BackArgs &b, int t, int tile) {
-    switch (algo) {
-        case PET_ALGO_OSEM: back_tile_body<EPI_OSEM, float, kRun, GENPOT>(b, t, tile); break;
-        case PET_ALGO_SVREM: back_tile_body<EPI_SVREM, float, kRun, GENPOT>(b, t, tile); break;
-        case PET_ALGO_SAGA:
-            if (table_dtype == PET_TABLE_BF16)
-                back_tile_body<EPI_SAGA, __nv_bfloat16, kRun, GENPOT>(b, t, tile);
-            else
-                back_tile_body<EPI_SAGA, float, kRun, GENPOT>(b, t, tile);
-            break;
-        case PET_ALGO_SGA: back_tile_body<EPI_SGA, float, kRun, GENPOT>(b, t, tile); break;
-        case PET_ALGO_SEM: back_tile_body<EPI_SEM, float, kRun, GENPOT>(b, t, tile); break;
-        case PET_ALGO_SAGAEM: back_tile_body<EPI_SAGAEM, float, kRun, GENPOT>(b, t, tile); break;
-        default: back_tile_body<EPI_SVRG, float, kRun, GENPOT>(b, t, tile); break;
-    }
+    back_run_body<EPI, TQ, GENPOT>(a, t, blockIdx.x);
 }
 
 // Persistent batched back projection + update: a resident grid whose blocks
 // claim work items until the list is exhausted.  An item is one tile of a
 // member's update (WK_BACK_UPDATE) or one (subset, tile) of a member's anchor
-// back projection (WK_BACK_ANCHOR), run by the same body with the same run
-// length as the member's own launches, so results are bit-identical to them.
+// back projection (WK_BACK_ANCHOR), run by the same body as the member's own
+// launches, so results are bit-identical to them.
 // Thread 0 claims the item and writes its arguments to shared memory; the
 // segment table is staged in shared memory once per block.
-// GENPOT: the members of this launch use an edge-preserving potential.
-template <bool GENPOT>
-__global__ void __maxnreg__(kPersistentBackRegs)
+// GENPOT: the members of this launch use an edge-preserving potential.  REF:
+// they are SAGA states with BF16 tables (kRefRounding).
+template <bool GENPOT, bool REF>
+__global__ void __launch_bounds__(REF ? kRunBlock : tile_threads(kPx), REF ? 5 : 8)
     persistent_back_kernel(const BatchMember *ms, const WorkSeg *segs, int n_segs, int n_items, int iter,
                            int in_is_img, int *claim) {
     __shared__ WorkSeg s_segs[kSegSmem];
     __shared__ BackArgs s_b;
-    __shared__ int s_item, s_t, s_tile, s_kind, s_shape, s_algo, s_tq;
+    __shared__ int s_item, s_t, s_tile, s_kind, s_algo;
     for (int i = threadIdx.x; i < n_segs && i < kSegSmem; i += blockDim.x) s_segs[i] = segs[i];
     const WorkSeg *tab = n_segs <= kSegSmem ? s_segs : segs;
     // the segment table and member descriptors were copied in before the
@@ -118,7 +97,9 @@ __global__ void __maxnreg__(kPersistentBackRegs)
                 b.nz = 1;
                 b.nb = m.nb;
                 b.ns = m.ns;
-                b.run = sg.shape;
+                b.bw = m.bw;
+                b.cand1 = m.cand1;
+                b.cand2 = m.cand2;
                 const int local = g - sg.first;
                 if (sg.kind == WK_BACK_ANCHOR) {
                     const int t = local / sg.tiles;
@@ -152,28 +133,43 @@ __global__ void __maxnreg__(kPersistentBackRegs)
                 }
                 s_b = b;
                 s_kind = sg.kind;
-                s_shape = sg.shape;
                 s_algo = m.algo;
-                s_tq = m.table_dtype;
             }
         }
         __syncthreads();
         if (s_item >= n_items) break;
         const int t = s_t, tile = s_tile;
-        if (s_kind == WK_BACK_ANCHOR) {
-            if (s_shape == 4)
-                back_tile_body<EPI_ANCHOR, float, 4, false>(s_b, t, tile);
-            else
-                back_tile_body<EPI_ANCHOR, float, 8, false>(s_b, t, tile);
-        } else if (s_shape == 4) {
-            member_update_tile<4, GENPOT>(s_algo, s_tq, s_b, t, tile);
+        if constexpr (REF) {
+            back_run_body<EPI_SAGA, __nv_bfloat16, GENPOT>(s_b, t, tile);
         } else {
-            member_update_tile<8, GENPOT>(s_algo, s_tq, s_b, t, tile);
+            if (s_kind == WK_BACK_ANCHOR)
+                back_tile_body<EPI_ANCHOR, float, false, kPx>(s_b, t, tile);
+            else
+                member_update_tile<GENPOT, kPx>(s_algo, s_b, t, tile);
         }
     }
 }
 
-size_t back_smem_bytes() { return (size_t)kChunk * (kTile * kTile * sizeof(float) + sizeof(ViewParams) + sizeof(int)); }
+// Dynamic shared memory (at least `base` bytes) that a subset launch of `blocks`
+// blocks asks for to bound how many of them an SM holds.  A dependent launch's
+// blocks are placed while the kernel ahead still runs, and pile up on the SMs
+// that have room, up to the register limit of four, while others stay empty:
+// the fullest SM sets the time.  Bounded to one above the even share; a tighter
+// bound (256^2: 131 us a SAGA epoch instead of 140) costs launches of several
+// streams more (the four-method step 1969 us instead of 1800), none 153 and
+// 1750 us; at an even share of three and more the register limit does.
+size_t residency_smem(const void *kernel, int blocks, size_t base) {
+    const int cap = (blocks + sm_count() - 1) / sm_count() + 1;
+    if (cap > 3) return base;
+    constexpr size_t kPerSm = 227 << 10, kReserved = 1 << 10;     // shared memory of an SM; a block's own overhead
+    const size_t need = kPerSm / (size_t)(cap + 1) - kReserved + 1024;
+    if (need <= base ||
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need) != cudaSuccess) {
+        cudaGetLastError();
+        return base;
+    }
+    return need;
+}
 
 // Single-slice back-projection launch of one epilogue / table type / potential.
 struct TileBack {
@@ -186,45 +182,71 @@ struct TileBack {
     pet_status run() const {
         const int tiles = ((a.nx + kTile - 1) / kTile) * ((a.ny + kTile - 1) / kTile);
         const dim3 grid((unsigned)tiles, (unsigned)ny_grid);
-        const size_t smem = back_smem_bytes();
-        // one thread per run: kTile * kTile / run runs per view of the largest chunk
-        const int run = a.run == 4 ? 4 : 8;
-        const int per_view = kTile * (kTile / run);
-        // subset launches are latency-bound: one run per thread; the all-subset and
-        // full-data launches are throughput-bound: 256-thread blocks whose threads
-        // loop over the runs, so that more blocks fit per SM (anchor 41.3 -> 39.5 us)
-        const int threads = (wide_epilogue(EPI) && EPI != EPI_PLAIN)
-                                ? kTile * kTile
-                                : max(kTile * kTile, per_view * min(max_views, kChunk));
-        void (*k)(BackArgs) = nullptr;
-        if constexpr (wide_epilogue(EPI))
-            k = run == 4 ? back_tile_wide_kernel<EPI, TQ, 4, GENPOT> : back_tile_wide_kernel<EPI, TQ, 8, GENPOT>;
-        else
-            k = run == 4 ? back_tile_kernel<EPI, TQ, 4, GENPOT> : back_tile_kernel<EPI, TQ, 8, GENPOT>;
-        launch_dependent(k,
-                         grid, dim3((unsigned)threads), smem, s, a);
+        constexpr bool bf16 = std::is_same<TQ, __nv_bfloat16>::value;
+        if constexpr (bf16 || EPI == EPI_ANCHOR) {
+            if (bf16 || a.ref) {
+                // subset launches are latency-bound: one run per thread; the all-subset
+                // ones are throughput-bound: threads loop over the runs, so that more
+                // blocks fit per SM
+                const int per_view = kTile * kTile / kRun;
+                const int threads = ny_grid > 1 ? kRunBlock : max(kRunBlock, per_view * min(max_views, kRunViews));
+                launch_dependent(back_run_kernel<EPI, TQ, GENPOT>, grid, dim3((unsigned)threads), run_smem_bytes(), s,
+                                 a);
+                return check_launch("back_run_kernel");
+            }
+        }
+        if constexpr (!bf16) {
+            if constexpr (EPI == EPI_ANCHOR || EPI == EPI_SAGA_INIT || EPI == EPI_SAGAEM_INIT) {
+                launch_dependent(back_tile_kernel<EPI, TQ, GENPOT, kPx>, grid, dim3(tile_threads(kPx)),
+                                 tile_smem_bytes(), s, a);
+                return check_launch("back_tile_kernel");
+            }
+            if constexpr (EPI == EPI_PLAIN || EPI == EPI_SEM_INIT)
+                if (max_views >= kManyViews) {
+                    launch_dependent(back_tile_kernel<EPI, TQ, GENPOT, kPx, kViewGroups>, grid,
+                                     dim3(tile_threads(kPx) * kViewGroups), tile_smem_bytes(), s, a);
+                    return check_launch("back_tile_kernel");
+                }
+            const auto k = back_tile_kernel<EPI, TQ, GENPOT, 1>;
+            const size_t smem = tile_smem_bytes();
+            launch_dependent(k, grid, dim3(tile_threads(1)),
+                             a.t_dev ? residency_smem((const void *)k, tiles, smem) : smem, s, a);
+        }
         return check_launch("back_tile_kernel");
     }
 };
 
 }  // namespace
 
-int back_block_threads(int run, int max_views) {
-    const int per_view = kTile * (kTile / (run == 4 ? 4 : 8));
-    return std::min(kPersistentBackMax, std::max(kTile * kTile, per_view * std::min(max_views, kChunk)));
+// Bins a tile stages per view.  Over the tile's kTile x kTile pixels the first
+// candidate moves by at most (kTile - 1) (|cos| + |sin|) <= sqrt(2) (kTile - 1)
+// pixel / bin, and a pair of pixels has at most (2 + |du|) |cos| or (1 + 2 |du|)
+// |cos|, both <= sqrt(5), pixel / bin + 1 of them; two entries are always read,
+// and the rest is margin for rounding (see tile_view).  Bin numbers of 2^20 and more are beyond what the
+// candidates' float positions resolve: such plans read their bins in place
+// (a value above kStageBins).
+void tile_bins(double pixel_mm, double bin_mm, int nb, int nx, int ny, int &bw, int &cand1, int &cand2) {
+    static_assert(kPx <= 2, "candidates of at most a pair of pixels");
+    const double ratio = pixel_mm / bin_mm;
+    const double eps = 1e-3 + 4e-7 * ((double)nb + nx + ny);
+    bw = kStageBins + 1;
+    cand1 = cand2 = kUnrolledCand + 1;
+    if (nb >= (1 << 20) || ratio > (double)kStageBins) return;
+    cand1 = std::max(2, (int)std::floor(1.41422 * ratio + 2.0 * eps) + 1);
+    cand2 = std::max(2, (int)std::floor(2.23607 * ratio + 2.0 * eps) + 1);
+    bw = std::min(kStageBins + 1, (int)std::ceil((kTile - 1) * 1.41422 * ratio) + cand2 + 4);
 }
 
 pet_status launch_persistent_back(const BatchMember *d_members, const WorkSeg *d_segs, int n_segs, int n_items,
-                                  int iter, int in_is_img, int *claim, bool general_potential, int threads,
-                                  cudaStream_t s) {
+                                  int iter, int in_is_img, int *claim, bool general_potential, bool ref, cudaStream_t s) {
     if (n_items <= 0) return PET_OK;
     void (*k)(const BatchMember *, const WorkSeg *, int, int, int, int, int *) =
-        general_potential ? persistent_back_kernel<true> : persistent_back_kernel<false>;
-    const size_t smem = back_smem_bytes();
-    if (threads < kTile * kTile || threads > kPersistentBackMax)
-        return set_error(PET_ERR_INVALID, "back: block size");
-    static int resident[2][kPersistentBackMax + 1] = {};   // blocks per SM by potential class and block size
-    int &per_sm = resident[general_potential ? 1 : 0][threads];
+        general_potential ? (ref ? persistent_back_kernel<true, true> : persistent_back_kernel<true, false>)
+                          : (ref ? persistent_back_kernel<false, true> : persistent_back_kernel<false, false>);
+    const size_t smem = ref ? run_smem_bytes() : tile_smem_bytes();
+    const int threads = ref ? kRunBlock : tile_threads(kPx);
+    static int resident[2][2] = {};   // blocks per SM by potential class and rounding
+    int &per_sm = resident[general_potential ? 1 : 0][ref ? 1 : 0];
     if (per_sm == 0 &&
         (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)k, threads, smem) != cudaSuccess ||
          per_sm < 1))

@@ -93,24 +93,6 @@ __device__ __forceinline__ void finish_pixel(const FinArgs &a, long long i) {
     }
 }
 
-template <int kRun, bool GENPOT>
-__device__ __forceinline__ void df_update_tile(int algo, int table_dtype, const BackArgs &b, int t, int tile) {
-    switch (algo) {
-        case PET_ALGO_OSEM: back_tile_body<EPI_OSEM, float, kRun, GENPOT, true>(b, t, tile); break;
-        case PET_ALGO_SVREM: back_tile_body<EPI_SVREM, float, kRun, GENPOT, true>(b, t, tile); break;
-        case PET_ALGO_SAGA:
-            if (table_dtype == PET_TABLE_BF16)
-                back_tile_body<EPI_SAGA, __nv_bfloat16, kRun, GENPOT, true>(b, t, tile);
-            else
-                back_tile_body<EPI_SAGA, float, kRun, GENPOT, true>(b, t, tile);
-            break;
-        case PET_ALGO_SGA: back_tile_body<EPI_SGA, float, kRun, GENPOT, true>(b, t, tile); break;
-        case PET_ALGO_SEM: back_tile_body<EPI_SEM, float, kRun, GENPOT, true>(b, t, tile); break;
-        case PET_ALGO_SAGAEM: back_tile_body<EPI_SAGAEM, float, kRun, GENPOT, true>(b, t, tile); break;
-        default: back_tile_body<EPI_SVRG, float, kRun, GENPOT, true>(b, t, tile); break;
-    }
-}
-
 template <bool GENPOT>
 __global__ void __maxnreg__(kDataflowRegs)
     dataflow_epoch_kernel(const BatchMember *ms, const DfSeg *segs, int n_segs, int n_items, int odd, int *done,
@@ -120,7 +102,7 @@ __global__ void __maxnreg__(kDataflowRegs)
         BackArgs b;
         FinArgs fin;
     } s_args;
-    __shared__ int s_item, s_seg, s_ok, s_kind, s_shape, s_bx, s_t, s_algo, s_tq;
+    __shared__ int s_item, s_seg, s_ok, s_kind, s_shape, s_bx, s_t, s_algo, s_ref;
     int *claim = done;             // done[0]: the claim counter; done[1 + k]: items of segment k done
     int *seg_done = done + 1;
     // the counters were zeroed by the kernel ahead of this one
@@ -151,7 +133,7 @@ __global__ void __maxnreg__(kDataflowRegs)
                     s_shape = sg.shape;
                     s_bx = local;
                     s_algo = m.algo;
-                    s_tq = m.table_dtype;
+                    s_ref = m.ref;
                     if (sg.kind == DF_FWD_UPDATE || sg.kind == DF_FWD_ANCHOR) {
                         FwdArgs a{};
                         a.views = m.views;
@@ -205,7 +187,9 @@ __global__ void __maxnreg__(kDataflowRegs)
                         b.nz = 1;
                         b.nb = m.nb;
                         b.ns = m.ns;
-                        b.run = sg.shape;
+                        b.bw = m.bw;
+                        b.cand1 = m.cand1;
+                        b.cand2 = m.cand2;
                         if (sg.kind == DF_BACK_ANCHOR) {
                             const int t = local / sg.tiles;
                             b.r = m.ratio_full;
@@ -245,19 +229,16 @@ __global__ void __maxnreg__(kDataflowRegs)
         if (s_ok) {
             const int kind = s_kind, shape = s_shape, bx = s_bx;
             if (kind == DF_FWD_UPDATE || kind == DF_FWD_ANCHOR) {
-                forward_item<FWD_RATIO, false, true, true>(s_args.f, shape, bx);
+                forward_item<FWD_RATIO, false, true>(s_args.f, shape, bx);
             } else if (kind == DF_FINISH) {
                 const long long i = (long long)bx * kBlock + threadIdx.x;
-                if (threadIdx.x < kBlock && i < s_args.fin.plane) finish_pixel(s_args.fin, i);
+                if (i < s_args.fin.plane) finish_pixel(s_args.fin, i);
             } else if (kind == DF_BACK_ANCHOR) {
-                if (shape == 4)
-                    back_tile_body<EPI_ANCHOR, float, 4, false, true>(s_args.b, s_t, bx);
-                else
-                    back_tile_body<EPI_ANCHOR, float, 8, false, true>(s_args.b, s_t, bx);
-            } else if (shape == 4) {
-                df_update_tile<4, GENPOT>(s_algo, s_tq, s_args.b, s_t, bx);
+                back_tile_body<EPI_ANCHOR, float, false, 1, true>(s_args.b, s_t, bx);
+            } else if (s_ref) {
+                back_run_body<EPI_SAGA, __nv_bfloat16, GENPOT, true>(s_args.b, s_t, bx);
             } else {
-                df_update_tile<8, GENPOT>(s_algo, s_tq, s_args.b, s_t, bx);
+                member_update_tile<GENPOT, 1, true>(s_algo, s_args.b, s_t, bx);
             }
         }
         __syncthreads();
@@ -268,27 +249,24 @@ __global__ void __maxnreg__(kDataflowRegs)
     }
 }
 
-size_t df_smem_bytes() { return (size_t)kChunk * (kTile * kTile * sizeof(float) + sizeof(ViewParams) + sizeof(int)); }
-
 }  // namespace
 
 pet_status launch_dataflow_epoch(const BatchMember *d_members, const DfSeg *d_segs, int n_segs, int n_items,
                                  int odd, int *d_done, int *d_status, long long wait_limit, bool general_potential,
-                                 int threads, cudaStream_t s) {
+                                 cudaStream_t s) {
     if (n_items <= 0) return PET_OK;
-    if (threads < kTile * kTile || threads > kPersistentBackMax)
-        return set_error(PET_ERR_INVALID, "dataflow: block size");
     void (*k)(const BatchMember *, const DfSeg *, int, int, int, int *, int *, long long) =
         general_potential ? dataflow_epoch_kernel<true> : dataflow_epoch_kernel<false>;
-    const size_t smem = df_smem_bytes();
-    static int resident[2][kPersistentBackMax + 1] = {};   // blocks per SM by potential class and block size
-    int &per_sm = resident[general_potential ? 1 : 0][threads];
+    const size_t smem = std::max(tile_smem_bytes(), run_smem_bytes());
+    static_assert(kRunBlock == kBlock, "one pixel per thread in both back projections");
+    static int resident[2] = {};   // blocks per SM by potential class
+    int &per_sm = resident[general_potential ? 1 : 0];
     if (per_sm == 0 &&
-        (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)k, threads, smem) != cudaSuccess ||
+        (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)k, kBlock, smem) != cudaSuccess ||
          per_sm < 1))
         per_sm = 1;
     const int grid = std::min(n_items, per_sm * sm_count());
-    launch_dependent(k, dim3((unsigned)grid), dim3((unsigned)threads), smem, s, d_members, d_segs, n_segs, n_items,
+    launch_dependent(k, dim3((unsigned)grid), dim3(kBlock), smem, s, d_members, d_segs, n_segs, n_items,
                      odd, d_done, d_status, wait_limit);
     return check_launch("dataflow_epoch_kernel");
 }

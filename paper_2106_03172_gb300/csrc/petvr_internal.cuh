@@ -9,6 +9,7 @@
 #include <cmath>
 #include <cstdint>
 #include <cstdlib>
+#include <mutex>
 #include <string>
 #include <utility>
 #include <vector>
@@ -359,7 +360,9 @@ struct BackArgs {
     const int *sub_off;   // view offsets of subsets in `order`
     int t0;               // subset of blockIdx.y == 0
     const int *t_dev;     // if set: the subset index is read here (grid.y must be 1)
-    int run;              // single-slice tile kernel: pixels per run (4 or 8)
+    int bw;               // single-slice tile kernel: bins staged per view of a tile (tile_bins)
+    int cand1, cand2;     // and the most candidate bins of a pixel, of a pair of pixels
+    int ref;              // single slices, EPI_ANCHOR: kRefRounding
     int r_view0;          // view position of r[0] (ignored when t_dev is set: r is
                           //   then the compact ratio of subset *t_dev)
     int nx, ny, nz, nb, ns;  // nz: image entries per pixel (slices, or layers when axial)
@@ -399,6 +402,7 @@ struct BatchMember {
     int nx, ny, nb, ns;
     unsigned nb_mul;       // division by nb (FwdArgs)
     int nb_shift;
+    int bw, cand1, cand2;  // back-projection tiles (BackArgs)
     const float *sens_t;
     const float *sens;
     const float *g;
@@ -450,7 +454,7 @@ struct WorkSeg {
     int kind;     // WorkKind
     int first;    // list index of the segment's first item
     int count;    // items in the segment
-    int shape;    // forward: band chunks per ray; back: pixels per run
+    int shape;    // forward: band chunks per ray
     int tiles;    // back: tiles per subset (anchor item = t * tiles + tile)
 };
 
@@ -475,7 +479,7 @@ struct DfSeg {
     int kind;     // DfKind
     int first;    // list index of the segment's first item
     int count;    // items in the segment
-    int shape;    // forward: band chunks per ray; back: pixels per run
+    int shape;    // forward: band chunks per ray
     int tiles;    // back: tiles per subset
     int iter;     // the update this stage belongs to
     int flag;     // DF_FINISH of SVREM: s_hat is initialised from this anchor
@@ -513,7 +517,8 @@ struct pet_plan {
     int max_sub_views;
     int device;
     int fwd_chunks = 0;             // single-slice forward: band chunks per ray (8, 16 or 32)
-    int back_run = 8;               // single-slice back projection: pixels per run (4 or 8)
+    int back_run = 8;               // the caller's choice (4 or 8); no launch shape depends on it
+    int bw = 0, cand1 = 0, cand2 = 0;   // single-slice back projection (BackArgs)
     unsigned nb_mul = 0;            // division of a ray index by nb (bins_division)
     int nb_shift = 0;
     std::vector<int> order;         // subset-major view order
@@ -527,6 +532,9 @@ struct pet_plan {
     int *d_all_off = nullptr;       // {0, na}
     float *d_sens_t = nullptr;      // [ns][N]
     float *d_sens = nullptr;        // [N]
+    mutable float *d_sens_t_ref = nullptr;   // [ns + 1][N]: d_sens_t and d_sens in the reference
+                                             //   rounding, once a state needs them
+    mutable std::mutex ref_mu;      // guards d_sens_t_ref
     float4 *d_lz = nullptr;         // multi-ring: axial table per line [view][bin][pair]
 };
 
@@ -587,8 +595,8 @@ struct pet_batch {
     struct Phase {
         int kind;                   // 0 forward, 1 back + update (GENPOT 0/1 in `genpot`), 2 anchor finishes
         int seg_off, n_segs, n_items;
-        int threads;                // back: block size
         int genpot;                 // back: general-potential epilogues
+        int ref;                    // back: members with the reference rounding
         int claim;                  // claim counter slot
     };
     std::vector<std::vector<Phase>> phases;   // [n_iter]
@@ -666,15 +674,14 @@ pet_status launch_count_nnz(const FwdArgs &a, unsigned long long *d_count, cudaS
 // ratio kinds (WK_FWD_UPDATE, WK_FWD_ANCHOR), true the log-likelihood kind.
 pet_status launch_persistent_forward(const BatchMember *d_members, const WorkSeg *d_segs, int n_segs, int n_items,
                                      int iter, int in_is_img, int *claim, bool objective, cudaStream_t s);
+void tile_bins(double pixel_mm, double bin_mm, int nb, int nx, int ny, int &bw, int &cand1, int &cand2);   // BackArgs
 pet_status launch_persistent_back(const BatchMember *d_members, const WorkSeg *d_segs, int n_segs, int n_items,
-                                  int iter, int in_is_img, int *claim, bool general_potential, int threads,
-                                  cudaStream_t s);
+                                  int iter, int in_is_img, int *claim, bool general_potential, bool ref, cudaStream_t s);
 pet_status launch_zero_ints(int *p, int n, cudaStream_t s);
 // Dependency-driven batched epoch (dataflow.cu): the whole list in one launch.
 pet_status launch_dataflow_epoch(const BatchMember *d_members, const DfSeg *d_segs, int n_segs, int n_items,
                                  int odd, int *d_done, int *d_status, long long wait_limit, bool general_potential,
-                                 int threads, cudaStream_t s);
-int back_block_threads(int run, int max_views);   // block size a back projection of this shape needs
+                                 cudaStream_t s);
 int sm_count();
 pet_status launch_batch_objective_finish(const BatchMember *d_members, int n_members, int pen_blocks,
                                          cudaStream_t s);
