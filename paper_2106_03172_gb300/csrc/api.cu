@@ -337,7 +337,7 @@ pet_status state_init(pet_state *st, cudaStream_t s) {
 pet_status warm_start_into(const pet_problem *p, float *d_img, float *alt, float *ratio, double *sums,
                            cudaStream_t s) {
     const pet_plan *pl = p->plan;
-    PET_TRY(launch_uniform_image(p, d_img, s, sums));
+    PET_TRY(launch_uniform_image(p, d_img, s, sums, ratio, (long long)max_sub_rays(pl) * sino_inner(pl)));
     return pingpong(d_img, alt, plane_of(pl), pl->ns, s, [&](int i, const float *in, float *outp) {
         PET_TRY(ratio_subset(p, in, i, ratio, s));
         BackArgs b = back_args(pl, ratio, i, false);

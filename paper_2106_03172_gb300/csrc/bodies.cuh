@@ -18,6 +18,8 @@ namespace {
 
 constexpr int kTile = 16;           // single slice: a block owns a kTile x kTile pixel tile
 
+constexpr int kSubsetBatch = 4;
+
 // The bands [kb, ke) of one ray from this thread, every fourth one from kb on:
 // sum of share times pixel, in units of the ray length per band.
 //
@@ -27,7 +29,7 @@ constexpr int kTile = 16;           // single slice: a block owns a kTile x kTil
 // pass 23.2 us and 14.4M warp instructions (33.2 us and 22.0M with floorf, the
 // comparison of both band ends and contiguous bands per lane), a subset pass
 // 6.9 us (7.9).
-template <bool COH>
+template <bool COH, int kBatch>
 __device__ __forceinline__ float walk_bands(const FwdArgs &a, const ViewParams &vp, float uf, int ui, float hm,
                                             int n_minor, int kb, int ke) {
     const int s_major = vp.col ? 1 : a.nx;
@@ -39,7 +41,6 @@ __device__ __forceinline__ float walk_bands(const FwdArgs &a, const ViewParams &
     // kBatch bands at a time: all their offsets and shares first, then the
     // loads, then the FMAs in band order, so that the loads of a batch are in
     // flight together.
-    constexpr int kBatch = 4;
     for (int k = kb; k < ke; k += 4 * kBatch) {
         // the batch's base position: the integer part of kc du goes into the
         // pixel index, so that what is left stays small and exact
@@ -216,7 +217,7 @@ __device__ __forceinline__ void forward_tile_body(const FwdArgs &a, const int bx
     float acc = 0.0f;
     if (kb < ke)
         acc = REF ? walk_bands_ref<COH>(a, vp, uf, ui, hm, n_minor, kb, ke)
-                  : walk_bands<COH>(a, vp, uf, ui, hm, n_minor, kb, ke);
+                  : walk_bands<COH, CHUNKS >= 32 ? kSubsetBatch : 4>(a, vp, uf, ui, hm, n_minor, kb, ke);
     // the 4 chunks of each ray in this warp, then the warps of its group
     acc += __shfl_xor_sync(0xffffffffu, acc, 8);
     acc += __shfl_xor_sync(0xffffffffu, acc, 16);
@@ -251,18 +252,12 @@ __device__ __forceinline__ void forward_tile_body(const FwdArgs &a, const int bx
             }
         }
     }
-    if (LL) {
-        __shared__ double dred[kBlock / 32];
+    // every ray of the block is finished in its first warp (RAYS <= 32): the FP64
+    // sums, slow on GB300 (2 lanes per SM and clock), stay there
+    if (LL && warp == 0) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) ll += __shfl_xor_sync(0xffffffffu, ll, o);
-        if (lane == 0) dred[warp] = ll;
-        __syncthreads();
-        if (tid == 0) {
-            double s = 0.0;
-#pragma unroll
-            for (int i = 0; i < kBlock / 32; ++i) s += dred[i];
-            a.ll_partials[bx] = s;
-        }
+        for (int o = RAYS / 2; o > 0; o >>= 1) ll += __shfl_xor_sync(0xffffffffu, ll, o);
+        if (lane == 0) a.ll_partials[bx] = ll;
     }
 }
 

@@ -29,7 +29,7 @@ namespace {
 constexpr int kFwdMinBlocks = 5;
 
 template <int CHUNKS, int MODE, bool LL, bool REF = false>
-__global__ void __launch_bounds__(kBlock, kFwdMinBlocks) forward_tile_kernel(const FwdArgs a) {
+__global__ void __launch_bounds__(kBlock, CHUNKS >= 32 ? kFwdMinBlocks : 5) forward_tile_kernel(const FwdArgs a) {
     forward_tile_body<CHUNKS, MODE, LL, REF>(a, blockIdx.x);
 }
 
