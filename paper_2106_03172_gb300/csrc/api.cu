@@ -181,7 +181,7 @@ pet_status ratio_subset(const pet_problem *p, const float *f, int t, float *rati
     a.w_scalar = p->w_scalar;
     a.out = ratio;
     a.status = p->d_status;
-    return launch_forward(a, FWD_RATIO, false, choose_group(pl), s, nullptr);
+    return launch_forward(a, FWD_RATIO, false, subset_group(pl), s, nullptr);
 }
 
 // Whether a state's projections keep the reference rounding (kRefRounding).
@@ -234,7 +234,7 @@ pet_status ratio_all(const pet_problem *p, const float *f, float *ratio, cudaStr
     a.out = ratio;
     a.status = p->d_status;
     a.ref = ref;
-    return launch_forward(a, FWD_RATIO, false, full_group(pl), s, nullptr);
+    return launch_forward(a, FWD_RATIO, false, full_group(pl, ref != 0), s, nullptr);
 }
 
 // n_iter updates with the iterate ping-ponging between the caller's image and
@@ -741,7 +741,7 @@ pet_status pet_forward(const pet_plan *pl, const float *d_img, const float *d_bg
     a.w = d_bg;
     a.w_scalar = bg;
     a.out = d_sino;
-    return launch_forward(a, FWD_YHAT, false, subset < 0 ? full_group(pl) : choose_group(pl), (cudaStream_t)stream,
+    return launch_forward(a, FWD_YHAT, false, subset < 0 ? full_group(pl) : subset_group(pl), (cudaStream_t)stream,
                           nullptr);
 }
 
@@ -967,7 +967,7 @@ pet_status enqueue_update(pet_state *st, int algo, const int *t_dev, const float
     a.out = st->ratio;
     a.status = p->d_status;
     a.ref = ref_rounding(st);
-    PET_TRY(launch_forward(a, FWD_RATIO, false, choose_group(pl), s, nullptr, max_sub_rays(pl)));
+    PET_TRY(launch_forward(a, FWD_RATIO, false, subset_group(pl, a.ref != 0), s, nullptr, max_sub_rays(pl)));
     BackArgs b = back_args(pl, st->ratio, 0, false);
     b.t_dev = t_dev;
     b.f = in;
@@ -1965,8 +1965,9 @@ void build_batch_phases(pet_batch *b, int n_iter, const std::vector<std::vector<
                 any = true;
                 fa.push_back({j, WK_FWD_ANCHOR, 0, forward_blocks(pl->M, 1, full_group(pl)), full_group(pl), 0});
             }
-            fu.push_back({j, WK_FWD_UPDATE, 0, forward_blocks(max_sub_rays(pl), 1, choose_group(pl)),
-                          choose_group(pl), 0});
+            const int sub = subset_group(pl, ref_rounding(b->states[j]) != 0);
+            fu.push_back({j, WK_FWD_UPDATE, 0, forward_blocks(max_sub_rays(pl), 1, sub),
+                          sub, 0});
         }
         // bands per chunk decide an item's length
         auto longer_fwd = [&](const WorkSeg &x, const WorkSeg &y) {
@@ -2041,8 +2042,9 @@ void build_batch_dataflow(pet_batch *b, int n_iter, const std::vector<std::vecto
                           st->algo == PET_ALGO_SVREM && !ready ? 1 : 0, ab, -1);
                 if (st->algo == PET_ALGO_SVREM) ready = true;
             }
-            const int f = add(DF_FWD_UPDATE, forward_blocks(max_sub_rays(pl), 1, choose_group(pl)),
-                              choose_group(pl), i, 0, prev_b, -1);
+            const int sub = subset_group(pl, ref_rounding(st) != 0);
+            const int f = add(DF_FWD_UPDATE, forward_blocks(max_sub_rays(pl), 1, sub),
+                              sub, i, 0, prev_b, -1);
             prev_b = add(DF_BACK_UPDATE, tiles, 0, i, 0, f, fin);
         }
     }

@@ -655,7 +655,8 @@ pet_status launch_forward(const FwdArgs &a, int mode, bool ll, int group, cudaSt
                           int *n_blocks_out, int rays_for_grid = -1);
 int forward_blocks(int n_rays, int nz, int group);
 int choose_group(const pet_plan *plan);
-int full_group(const pet_plan *plan);     // band chunks of a full-data single-slice pass
+int subset_group(const pet_plan *plan, bool ref = false);   // band chunks of subset passes
+int full_group(const pet_plan *plan, bool ref = false);     // and of full-data passes
 int default_chunks(int nx, int ny);
 pet_status launch_back(const BackArgs &a, int epi, int table_dtype, int n_subsets_grid,
                        cudaStream_t s, int max_views);
