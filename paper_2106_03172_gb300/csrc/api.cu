@@ -166,6 +166,8 @@ BackArgs back_args(const pet_plan *pl, const float *r, int subset, bool natural)
     a.bw = pl->bw;
     a.cand1 = pl->cand1;
     a.cand2 = pl->cand2;
+    a.cands = pl->cands;
+    a.cand_rounds = pl->cand_rounds;
     return a;
 }
 
@@ -467,6 +469,7 @@ pet_status pet_plan_create(const pet_geometry *g, const pet_subsets *sub, pet_pl
     pl->nb = g->n_bins;
     bins_division(pl->nb, pl->nb_mul, pl->nb_shift);
     tile_bins(g->pixel_mm, ds_chk, pl->nb, pl->nx, pl->ny, pl->bw, pl->cand1, pl->cand2);
+    stack_candidates(g->pixel_mm, ds_chk, pl->nb, pl->nx, pl->ny, pl->cands, pl->cand_rounds);
     pl->ns = sub->n_subsets;
     pl->N = (int)N;
     pl->M = (int)M;

@@ -208,6 +208,47 @@ __device__ __forceinline__ void stage_views(const BackArgs &a, int vb, int nv, V
     }
 }
 
+// Slice stacks: the pieces of a warp's list (offset, weight) times the values at base[i] +
+// offset, into sums of the even and the odd pieces: groups of 8 / W pieces, whose
+// loads are in flight together, then the rest as one group whose missing
+// pieces repeat the last one's load and are left out.
+template <int W>
+__device__ __forceinline__ void add_pieces(const float2 *piece, int np, const float *const (&base)[W],
+                                           float (&sum)[2][W]) {
+    constexpr int U = 8 / W;
+    int b = 0;
+#pragma unroll 1
+    for (; b + U <= np; b += U) {
+        float2 p[U];
+        float x[U][W];
+#pragma unroll
+        for (int u = 0; u < U; ++u) p[u] = piece[b + u];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int i = 0; i < W; ++i) x[u][i] = __ldg(base[i] + __float_as_int(p[u].x));
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int i = 0; i < W; ++i) sum[u & 1][i] = fmaf(p[u].y, x[u][i], sum[u & 1][i]);
+    }
+    if (b < np) {
+        float2 p[U];
+        float x[U][W];
+#pragma unroll
+        for (int u = 0; u < U; ++u) p[u] = piece[min(b + u, np - 1)];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int i = 0; i < W; ++i) x[u][i] = __ldg(base[i] + __float_as_int(p[u].x));
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (b + u < np)
+#pragma unroll
+                for (int i = 0; i < W; ++i) sum[u & 1][i] = fmaf(p[u].y, x[u][i], sum[u & 1][i]);
+    }
+}
+
 constexpr bool uses_stencil(int epi) {
     return epi == EPI_OSEM || epi == EPI_SVREM || epi == EPI_SAGA || epi == EPI_SAGA_INIT || epi == EPI_SVRG ||
            epi == EPI_SGA || epi == EPI_SEM || epi == EPI_SAGAEM;

@@ -328,15 +328,19 @@ __device__ __forceinline__ RayRange ray_range(const FwdArgs &a) {
     return r;
 }
 
-// Slice stacks (the geometry is shared by every slice): a warp of the forward
-// is kStackChunks band chunks x 8 z-lanes, one of the back projection
-// kStackPixels pixels x 8 z-lanes, and a z-lane carries stack_lane_slices(nz)
-// slices (a window of 8 times that many per warp; deeper stacks take several
-// windows).
+// Slice stacks (the geometry is shared by every slice).  Up to kSlimSlices
+// slices: a warp of the forward is kStackChunks band chunks x 8 z-lanes, one of
+// the back projection kStackPixels pixels x 8 z-lanes, and a z-lane carries every
+// eighth slice.  Deeper stacks: a warp takes one ray (pixel) and a window of 32
+// stack_lane_slices(nz) slices, every lane its own slices.
 constexpr int kStackChunks = 4;
 constexpr int kStackPixels = 4;
-inline int stack_lane_slices(int nz) { return nz <= 16 ? 2 : nz <= 32 ? 4 : nz <= 48 ? 6 : 8; }
-inline int stack_windows(int nz) { return (nz + 8 * stack_lane_slices(nz) - 1) / (8 * stack_lane_slices(nz)); }
+constexpr int kSlimSlices = 16;
+inline int stack_lane_slices(int nz) { return nz <= kSlimSlices ? 0 : nz <= 32 ? 1 : 2; }
+inline int stack_windows(int nz) {
+    const int per = nz <= kSlimSlices ? kSlimSlices : 32 * stack_lane_slices(nz);
+    return (nz + per - 1) / per;
+}
 
 enum BackEpi {
     EPI_PLAIN = 0,       // out = A_t^T r
@@ -362,6 +366,7 @@ struct BackArgs {
     const int *t_dev;     // if set: the subset index is read here (grid.y must be 1)
     int bw;               // single-slice tile kernel: bins staged per view of a tile (tile_bins)
     int cand1, cand2;     // and the most candidate bins of a pixel, of a pair of pixels
+    int cands, cand_rounds;   // slice stacks: lanes per view, 32-bin pieces per view
     int ref;              // single slices, EPI_ANCHOR: kRefRounding
     int r_view0;          // view position of r[0] (ignored when t_dev is set: r is
                           //   then the compact ratio of subset *t_dev)
@@ -519,6 +524,7 @@ struct pet_plan {
     int fwd_chunks = 0;             // single-slice forward: band chunks per ray (8, 16 or 32)
     int back_run = 8;               // the caller's choice (4 or 8); no launch shape depends on it
     int bw = 0, cand1 = 0, cand2 = 0;   // single-slice back projection (BackArgs)
+    int cands = 1, cand_rounds = 1;     // slice stacks (BackArgs)
     unsigned nb_mul = 0;            // division of a ray index by nb (bins_division)
     int nb_shift = 0;
     std::vector<int> order;         // subset-major view order
@@ -648,6 +654,8 @@ bool profiling_enabled();
 // Kernel launchers (forward.cu / backward.cu / misc.cu).
 // Volumes (volume.cu): slice stacks and multi-ring scanners.
 pet_status launch_forward_volume(const FwdArgs &a, int mode, bool ll, int group, int blocks, cudaStream_t s);
+// Candidate bins of a pixel (candidate_bins) as lanes per view, at most 32, and 32-bin pieces.
+void stack_candidates(double pixel_mm, double bin_mm, int nb, int nx, int ny, int &cands, int &rounds);
 pet_status launch_back_volume(const BackArgs &a, int epi, int table_dtype, int n_subsets_grid, cudaStream_t s,
                               int max_views);
 pet_status launch_count_nnz_ring(const FwdArgs &a, unsigned long long *d_count, cudaStream_t s);

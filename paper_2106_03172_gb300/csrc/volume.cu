@@ -9,8 +9,24 @@ namespace petvr {
 
 namespace {
 
-// Slice-stack forward: the geometry is shared by every slice.  A warp takes
-// one ray and a window of 8 ZW consecutive slices; its lanes are kStackChunks
+// One block's sum of the log-likelihood terms (FP64; kBlock threads): the terms
+// meet in shared memory and one warp adds them, since FP64 runs at 2 lanes per
+// SM and clock.
+__device__ __forceinline__ void block_ll(double ll, double *partials) {
+    __shared__ double s_ll[kBlock];
+    s_ll[threadIdx.x] = ll;
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    double s = 0.0;
+#pragma unroll
+    for (int i = 0; i < kBlock / 32; ++i) s += s_ll[threadIdx.x + 32 * i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) partials[blockIdx.x] = s;
+}
+
+// Slice-stack forward of at most kSlimSlices slices: a warp takes one ray and
+// all slices (ZW = kSlimSlices / 8); its lanes are kStackChunks
 // band chunks x 8 z-lanes, and z-lane l carries slices l, l + 8, ... of the
 // window, so each load instruction reads 8 consecutive floats of a pixel's
 // slice column per chunk ([iy][ix][z] layout: coalesced).  The band geometry
@@ -20,7 +36,7 @@ namespace {
 // then w1 piece) and the chunk sums are combined by xor-shuffles in a fixed
 // order, so the result is deterministic.
 template <int MODE, bool LL, int ZW>
-__global__ void __launch_bounds__(kBlock) forward_stack_kernel(const FwdArgs a) {
+__global__ void __launch_bounds__(kBlock) forward_slim_kernel(const FwdArgs a) {
     const RayRange rr = ray_range(a);
     // 32-bit index arithmetic: images and sinograms are below 2^31 elements (checked at plan time)
     const int n_rays = (rr.v_end - rr.v_begin) * a.nb;
@@ -129,19 +145,114 @@ __global__ void __launch_bounds__(kBlock) forward_stack_kernel(const FwdArgs a) 
             }
         }
     }
-    if (LL) {
-        __shared__ double red[kBlock / 32];
+    if (LL) block_ll(ll, a.ll_partials);
+}
+
+// Slice-stack forward: the geometry is shared by every slice.  A warp takes one
+// ray and a window of 32 W consecutive slices, lane l the slices l, l + 32, ...
+// of the window, so a load instruction reads 32 consecutive floats of one
+// pixel's slice column ([iy][ix][z] layout).  For kStackBands bands of the ray at
+// a time, lane l evaluates the bands l, l + 32, ... once for all slices, and the
+// nonzero pieces go to a list in shared memory, in band order, which the warp
+// then walks (the same pieces for every lane) into two sums, even and odd
+// pieces (deterministic).
+//
+// Bound by instruction issue (seven instructions per piece and two windows of
+// slices) and the gathers' L1 wavefronts.  47 slices of 128^2, 252 views of 344
+// bins (ncu), against 8 z-lanes x 4 chunks (forward_slim_kernel's layout): full
+// ratio pass 263 -> 170 us (183M -> 118M warp instructions, L1 wavefronts 85% ->
+// 66%), a subset 29.4 -> 22.1 us.
+constexpr int kStackBands = 128;
+
+template <int MODE, bool LL, int W>
+__global__ void __launch_bounds__(kBlock, 4) forward_stack_kernel(const FwdArgs a) {
+    __shared__ float2 s_piece[kBlock / 32][2 * kStackBands];   // image offset, weight
+    const RayRange rr = ray_range(a);
+    // 32-bit index arithmetic: images and sinograms are below 2^31 elements (checked at plan time)
+    const int n_rays = (rr.v_end - rr.v_begin) * a.nb;
+    const int n_win = (a.nz + 32 * W - 1) / (32 * W);
+    const int lane = threadIdx.x & 31;
+    float2 *piece = s_piece[threadIdx.x >> 5];
+    const long long wid = (long long)blockIdx.x * (kBlock / 32) + (threadIdx.x >> 5);
+    const int ray = n_win == 1 ? (int)min(wid, (long long)n_rays) : (int)min(wid / n_win, (long long)n_rays);
+    const int win = n_win == 1 ? 0 : (int)(wid % n_win);
+    const bool live = ray < n_rays;                       // the same for the whole warp
+    const int z0 = win * 32 * W + lane;                   // this lane's first slice
+
+    float sum[2][W] = {};
+    if (live) {
+        const int q = div_by_bins(ray, a.nb_mul, a.nb_shift);
+        const int j = ray - q * a.nb;
+        const int v = __ldg(a.order + rr.v_begin + q);
+        const ViewParams vp = a.views[v];
+        const float2 u = __ldg(a.uc + v * a.nb + j);
+        const int n_major = vp.col ? a.nx : a.ny;
+        const int n_minor = vp.col ? a.ny : a.nx;
+        const float hm = 0.5f * (float)n_major;
+        int k_lo, k_hi;
+        band_range(vp, u.x + u.y, n_major, n_minor, k_lo, k_hi);
+        const int s_major = (vp.col ? 1 : a.nx) * a.nz;   // strides of a pixel's slice column
+        const int s_minor = (vp.col ? a.nx : 1) * a.nz;
+        const int ui = (int)u.x + (n_minor >> 1);         // pixel index of fractional position 0
+        // a lane past the last slice reads that slice again and drops the sum
+        const float *img[W];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) ll += __shfl_xor_sync(0xffffffffu, ll, o);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ll;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double sum = 0.0;
-#pragma unroll
-            for (int i = 0; i < kBlock / 32; ++i) sum += red[i];
-            a.ll_partials[blockIdx.x] = sum;
+        for (int i = 0; i < W; ++i) img[i] = a.img + min(z0 + 32 * i, a.nz - 1);
+        for (int kseg = k_lo; kseg < k_hi; kseg += kStackBands) {
+            const int ke = min(k_hi, kseg + kStackBands);
+            int np = 0;
+            __syncwarp();
+            for (int kbase = kseg; kbase < ke; kbase += 32) {
+                const int k = kbase + lane;
+                float w0 = 0.0f, w1 = 0.0f;
+                int o = 0;
+                if (k < ke) {
+                    const float kc = (float)k - hm;
+                    const float t = band_split_ref(vp, band_point(vp, u.y, kc), band_point(vp, u.y, kc + 1.0f), w0, w1);
+                    const int m0 = (int)(__float_as_uint(t) - kRoundBits) + ui;
+                    o = k * s_major + m0 * s_minor;
+                    if ((unsigned)m0 >= (unsigned)n_minor) w0 = 0.0f;
+                    if (!(w1 > 0.0f) || (unsigned)(m0 + 1) >= (unsigned)n_minor) w1 = 0.0f;
+                }
+                const unsigned has0 = __ballot_sync(0xffffffffu, w0 != 0.0f), has1 = __ballot_sync(0xffffffffu, w1 != 0.0f);
+                const unsigned before = (1u << lane) - 1;
+                int at = np + __popc(has0 & before) + __popc(has1 & before);
+                if (w0 != 0.0f) piece[at++] = make_float2(__int_as_float(o), w0);
+                if (w1 != 0.0f) piece[at] = make_float2(__int_as_float(o + s_minor), w1);
+                np += __popc(has0) + __popc(has1);
+            }
+            __syncwarp();
+            add_pieces<W>(piece, np, img, sum);
         }
     }
+
+    double ll = 0.0;
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+        if (!live || z0 + 32 * i >= a.nz) continue;
+        const int idx = ray * a.nz + z0 + 32 * i;
+        const long long gi = rr.off + idx;
+        const float yhat = (sum[0][i] + sum[1][i]) + (a.w ? __ldg(a.w + gi) : a.w_scalar);
+        if (MODE == FWD_YHAT) a.out[idx] = yhat;
+        if (MODE == FWD_RATIO || LL) {
+            const float g = __ldg(a.g + gi);
+            if (MODE == FWD_RATIO) a.out[idx] = (yhat != 0.0f) ? g / yhat : 0.0f;
+            if (LL) {
+                if (yhat > 0.0f) {
+                    // per-ray term with an FP32 log (GB300's FP64 pipe is too slow for a
+                    // log per ray; the term's error, ~g ulp(log yhat), is far below the
+                    // FP32 rounding of yhat itself), reduced in FP64
+                    ll += (g > 0.0f ? (double)g * (double)logf(yhat) : 0.0) - (double)yhat;
+                } else if (g > 0.0f) {
+                    ll = -(double)INFINITY;            // log of a nonpositive mean: Phi = -inf
+                    if (a.status) atomicExch(a.status, (int)PET_ERR_NUMERIC);
+                } else {
+                    ll += -(double)yhat;
+                }
+            }
+        }
+    }
+    if (LL) block_ll(ll, a.ll_partials);
 }
 
 // Multi-ring forward: CH consecutive lanes per ray, each walking one chunk of
@@ -251,19 +362,7 @@ __global__ void __launch_bounds__(kBlock) ring_forward_kernel(const FwdArgs a) {
             }
         }
     }
-    if (LL) {
-        __shared__ double red[kBlock / 32];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) ll += __shfl_xor_sync(0xffffffffu, ll, o);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ll;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double sum = 0.0;
-#pragma unroll
-            for (int i = 0; i < kBlock / 32; ++i) sum += red[i];
-            a.ll_partials[blockIdx.x] = sum;
-        }
-    }
+    if (LL) block_ll(ll, a.ll_partials);
 }
 
 // Nonzeros of the multi-ring lines of a view range: (piece, layer) pairs of
@@ -336,27 +435,28 @@ pet_status dispatch_ring(const FwdArgs &a, int mode, bool ll, int blocks, cudaSt
     }
 }
 
-template <int ZW>
-pet_status dispatch_stack_zw(const FwdArgs &a, int mode, bool ll, int blocks, cudaStream_t s) {
+template <int W>
+pet_status dispatch_stack_w(const FwdArgs &a, int mode, bool ll, int blocks, cudaStream_t s) {
+    void (*k)(FwdArgs) = nullptr;
     if (mode == FWD_YHAT && !ll)
-        forward_stack_kernel<FWD_YHAT, false, ZW><<<blocks, kBlock, 0, s>>>(a);
+        k = W ? forward_stack_kernel<FWD_YHAT, false, W ? W : 1> : forward_slim_kernel<FWD_YHAT, false, kSlimSlices / 8>;
     else if (mode == FWD_RATIO && !ll)
-        forward_stack_kernel<FWD_RATIO, false, ZW><<<blocks, kBlock, 0, s>>>(a);
+        k = W ? forward_stack_kernel<FWD_RATIO, false, W ? W : 1> : forward_slim_kernel<FWD_RATIO, false, kSlimSlices / 8>;
     else if (mode == FWD_RATIO && ll)
-        forward_stack_kernel<FWD_RATIO, true, ZW><<<blocks, kBlock, 0, s>>>(a);
+        k = W ? forward_stack_kernel<FWD_RATIO, true, W ? W : 1> : forward_slim_kernel<FWD_RATIO, true, kSlimSlices / 8>;
     else if (mode == FWD_NONE && ll)
-        forward_stack_kernel<FWD_NONE, true, ZW><<<blocks, kBlock, 0, s>>>(a);
+        k = W ? forward_stack_kernel<FWD_NONE, true, W ? W : 1> : forward_slim_kernel<FWD_NONE, true, kSlimSlices / 8>;
     else
         return set_error(PET_ERR_INVALID, "forward: unsupported mode");
+    k<<<blocks, kBlock, 0, s>>>(a);
     return check_launch("forward_stack_kernel");
 }
 
 pet_status dispatch_stack(const FwdArgs &a, int mode, bool ll, int blocks, cudaStream_t s) {
     switch (stack_lane_slices(a.nz)) {
-        case 2: return dispatch_stack_zw<2>(a, mode, ll, blocks, s);
-        case 4: return dispatch_stack_zw<4>(a, mode, ll, blocks, s);
-        case 6: return dispatch_stack_zw<6>(a, mode, ll, blocks, s);
-        default: return dispatch_stack_zw<8>(a, mode, ll, blocks, s);
+        case 0: return dispatch_stack_w<0>(a, mode, ll, blocks, s);
+        case 1: return dispatch_stack_w<1>(a, mode, ll, blocks, s);
+        default: return dispatch_stack_w<2>(a, mode, ll, blocks, s);
     }
 }
 

@@ -4,6 +4,9 @@
 // update as the single-slice kernels (epilogue.cuh).  The multi-ring weights
 // come from the expressions the forward projector uses (piece_fraction /
 // piece_zeta / layer_fraction), so A^T is the exact transpose of A.
+#include <algorithm>
+#include <cmath>
+
 #include "epilogue.cuh"
 
 namespace petvr {
@@ -21,7 +24,7 @@ namespace {
 // a shuffle; views and candidates are added in order (deterministic).  Each
 // lane then applies the update to its own slices.
 template <int EPI, typename TQ, bool GENPOT, int ZW>
-__global__ void __launch_bounds__(kBlock) back_stack_kernel(const BackArgs a) {
+__global__ void __launch_bounds__(kBlock) back_slim_kernel(const BackArgs a) {
     extern __shared__ unsigned char smem_raw[];
     ViewParams *s_views = reinterpret_cast<ViewParams *>(smem_raw);
     const int t = a.t_dev ? __ldg(a.t_dev) : a.t0 + (int)blockIdx.y;
@@ -93,6 +96,96 @@ __global__ void __launch_bounds__(kBlock) back_stack_kernel(const BackArgs a) {
             const int z = z0 + 8 * i;
             apply_epilogue<EPI, TQ, GENPOT>(a, t, (long long)n * a.nz + z, n, ix, iy, z, acc[i]);
         }
+}
+
+// Slice-stack path: the geometry is shared by every slice.  A warp takes one
+// pixel and a window of 32 W consecutive slices, lane l the slices l, l + 32,
+// ... of the window, so a load instruction reads 32 consecutive floats of one
+// bin's slice column ([view][bin][z]).  The lanes share the candidate bins of
+// the subset's views among them (a.cands per view), evaluate each one's band
+// piece once for all slices, and leave the nonzero weights, in view and bin
+// order, in shared memory; the warp then walks that list into two sums, even and
+// odd pieces (deterministic), and each lane applies the update to its own
+// slices.  Bound by instruction issue.  47 slices of 128^2 (ncu), against 4
+// pixels x 8 z-lanes (back_slim_kernel's layout): anchor of 14 subsets 290 -> 231
+// us, an update 37.5 -> 32.1 us; 24 slices of 96^2, a run call 723 -> 440 us.
+constexpr int kStackPieces = 96;     // list entries per warp (a round adds up to 32)
+
+template <int EPI, typename TQ, bool GENPOT, int W>
+__global__ void __launch_bounds__(kBlock, 5) back_stack_kernel(const BackArgs a) {
+    extern __shared__ unsigned char smem_raw[];
+    __shared__ float2 s_piece[kBlock / 32][kStackPieces];   // ratio offset, weight
+    ViewParams *s_views = reinterpret_cast<ViewParams *>(smem_raw);
+    const int t = a.t_dev ? __ldg(a.t_dev) : a.t0 + (int)blockIdx.y;
+    const int vb = __ldg(a.sub_off + t);
+    const int nv = __ldg(a.sub_off + t + 1) - vb;
+    int *s_vid = reinterpret_cast<int *>(s_views + nv);
+    stage_views(a, vb, nv, s_views, s_vid);
+    __syncthreads();
+    const int r_view0 = a.t_dev ? vb : a.r_view0;
+
+    // 32-bit index arithmetic: images and sinograms are below 2^31 elements (checked at plan time)
+    const int n_win = (a.nz + 32 * W - 1) / (32 * W);
+    const int lane = threadIdx.x & 31;
+    float2 *piece = s_piece[threadIdx.x >> 5];
+    const int wid = blockIdx.x * (kBlock / 32) + (threadIdx.x >> 5);
+    const int n = n_win == 1 ? wid : wid / n_win;         // pixel
+    const int win = n_win == 1 ? 0 : wid - n * n_win;
+    if (n >= a.nx * a.ny) return;                         // the whole warp
+    const int ix = n % a.nx;
+    const int iy = n / a.nx;
+    const int z0 = win * 32 * W + lane;                   // this lane's first slice
+
+    float acc[2][W] = {};
+    // a lane past the last slice reads that slice again and drops the sum
+    const float *r[W];
+#pragma unroll
+    for (int i = 0; i < W; ++i) r[i] = a.r + min(z0 + 32 * i, a.nz - 1);
+    // views per round; a view with more than 32 candidates takes cand_rounds rounds
+    const int per_round = 32 / a.cands;
+    const int rounds = (nv + per_round - 1) / per_round * a.cand_rounds;
+    const int lq = lane / a.cands, lc = lane - lq * a.cands;
+    int np = 0;
+    for (int round = 0; round < rounds; ++round) {
+        const int part = a.cand_rounds == 1 ? 0 : round % a.cand_rounds;
+        const int q = (a.cand_rounds == 1 ? round : round / a.cand_rounds) * per_round + lq;
+        float w = 0.0f;
+        int off = 0;
+        if (lq < per_round && q < nv) {
+            const ViewParams vp = s_views[q];
+            const int k = vp.col ? ix : iy;              // major index
+            const int minor = vp.col ? iy : ix;
+            const int n_major = vp.col ? a.nx : a.ny;
+            const int n_minor = vp.col ? a.ny : a.nx;
+            const int mrel = minor - (n_minor >> 1);
+            const float kc = (float)k - 0.5f * (float)n_major;
+            int jlo, jhi;
+            candidate_bins(vp, kc, (float)mrel, (float)mrel + 1.0f, a.nb, jlo, jhi);
+            const int j = jlo + lc + 32 * part;
+            if (j <= jhi) {
+                const float2 u = __ldg(a.uc + s_vid[q] * a.nb + j);
+                float w0, w1;
+                const float t = band_split_ref(vp, band_point(vp, u.y, kc), band_point(vp, u.y, kc + 1.0f), w0, w1);
+                const int c0 = (int)(__float_as_uint(t) - kRoundBits) + (int)u.x;
+                w = (c0 == mrel) ? w0 : ((c0 + 1 == mrel) ? w1 : 0.0f);
+                off = ((vb + q - r_view0) * a.nb + j) * a.nz;
+            }
+        }
+        const unsigned mask = __ballot_sync(0xffffffffu, w != 0.0f);
+        if (w != 0.0f) piece[np + __popc(mask & ((1u << lane) - 1))] = make_float2(__int_as_float(off), w);
+        np += __popc(mask);
+        if (np <= kStackPieces - 32 && round + 1 < rounds) continue;     // room for another round
+        __syncwarp();
+        add_pieces<W>(piece, np, r, acc);
+        __syncwarp();
+        np = 0;
+    }
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+        const int z = z0 + 32 * i;
+        if (z < a.nz)
+            apply_epilogue<EPI, TQ, GENPOT>(a, t, (long long)n * a.nz + z, n, ix, iy, z, acc[0][i] + acc[1][i]);
+    }
 }
 
 // Multi-ring path: kLanes lanes per voxel share the subset's views (lane l
@@ -280,22 +373,32 @@ struct VolumeBack {
             ring_back_kernel<EPI, TQ, GENPOT><<<grid, kBlock, smem, s>>>(a);
             return check_launch("ring_back_kernel");
         }
-        // one warp per kStackPixels pixels and slice window
-        const int zw = stack_lane_slices(a.nz);
-        const long long quads = ((long long)a.nx * a.ny + kStackPixels - 1) / kStackPixels;
-        const long long warps = quads * stack_windows(a.nz);
+        const int w = stack_lane_slices(a.nz);
+        const long long pixels = (long long)a.nx * a.ny;
+        // one warp per kStackPixels pixels, or per pixel and slice window
+        const long long warps = w == 0 ? (pixels + kStackPixels - 1) / kStackPixels : pixels * stack_windows(a.nz);
         const dim3 grid((unsigned)((warps + kBlock / 32 - 1) / (kBlock / 32)), (unsigned)ny_grid);
-        switch (zw) {
-            case 2: back_stack_kernel<EPI, TQ, GENPOT, 2><<<grid, kBlock, smem, s>>>(a); break;
-            case 4: back_stack_kernel<EPI, TQ, GENPOT, 4><<<grid, kBlock, smem, s>>>(a); break;
-            case 6: back_stack_kernel<EPI, TQ, GENPOT, 6><<<grid, kBlock, smem, s>>>(a); break;
-            default: back_stack_kernel<EPI, TQ, GENPOT, 8><<<grid, kBlock, smem, s>>>(a); break;
+        switch (w) {
+            case 0: back_slim_kernel<EPI, TQ, GENPOT, kSlimSlices / 8><<<grid, kBlock, smem, s>>>(a); break;
+            case 1: back_stack_kernel<EPI, TQ, GENPOT, 1><<<grid, kBlock, smem, s>>>(a); break;
+            default: back_stack_kernel<EPI, TQ, GENPOT, 2><<<grid, kBlock, smem, s>>>(a); break;
         }
         return check_launch("back_stack_kernel");
     }
 };
 
 }  // namespace
+
+// candidate_bins() gives the bins whose positions lie in a range of (1 + |du| +
+// 2 kCandEps) |cos| <= sqrt(2) + 2 kCandEps pixels, over bin spacings; the rest
+// is margin for the positions' rounding.
+void stack_candidates(double pixel_mm, double bin_mm, int nb, int nx, int ny, int &cands, int &rounds) {
+    const double ratio = pixel_mm / bin_mm;
+    const double most = (1.41422 + 2.0 * kCandEps) * ratio + 1e-2 + 2e-6 * ((double)nb + nx + ny);
+    const int n = most < nb ? (int)std::floor(most) + 1 : nb;
+    cands = std::min(n, 32);
+    rounds = (n + 31) / 32;
+}
 
 pet_status launch_back_volume(const BackArgs &a, int epi, int table_dtype, int n_subsets_grid, cudaStream_t s,
                               int max_views) {
