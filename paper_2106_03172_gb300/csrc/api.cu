@@ -164,8 +164,7 @@ BackArgs back_args(const pet_plan *pl, const float *r, int subset, bool natural)
     a.sens_t = pl->d_sens_t;
     a.sens = pl->d_sens;
     a.bw = pl->bw;
-    a.cand1 = pl->cand1;
-    a.cand2 = pl->cand2;
+    a.cand = pl->cand;
     a.cands = pl->cands;
     a.cand_rounds = pl->cand_rounds;
     return a;
@@ -183,51 +182,11 @@ pet_status ratio_subset(const pet_problem *p, const float *f, int t, float *rati
     a.w_scalar = p->w_scalar;
     a.out = ratio;
     a.status = p->d_status;
-    return launch_forward(a, FWD_RATIO, false, subset_group(pl), s, nullptr);
-}
-
-// Whether a state's projections keep the reference rounding (kRefRounding).
-int ref_rounding(const pet_state *st) {
-    const pet_plan *pl = st->prob->plan;
-    return st->algo == PET_ALGO_SAGA && st->table_dtype == PET_TABLE_BF16 && pl->nz == 1 && !pl->ring ? 1 : 0;
-}
-
-// Sensitivities of the reference rounding, of every subset and their sum (a
-// state's gradient subtracts the sensitivity of its own projector: other
-// rounding there would not cancel).  Made when the first state that needs them is, and kept by the plan.
-pet_status ensure_ref_sensitivity(const pet_plan *pl, cudaStream_t s) {
-    std::lock_guard<std::mutex> lk(pl->ref_mu);
-    if (pl->d_sens_t_ref) return PET_OK;
-    float *ones = nullptr, *sens = nullptr;
-    pet_status st = dalloc(&ones, (size_t)pl->M, "ones");
-    if (st == PET_OK) st = dalloc(&sens, (size_t)(pl->ns + 1) * pl->N, "reference sensitivities");
-    if (st == PET_OK) {
-        const std::vector<float> h1((size_t)pl->M, 1.0f);
-        st = cuda_ok(cudaMemcpyAsync(ones, h1.data(), sizeof(float) * pl->M, cudaMemcpyHostToDevice, s), "ones upload");
-        if (st == PET_OK) {
-            BackArgs b = back_args(pl, ones, -1, false);
-            b.t0 = 0;
-            b.r_view0 = 0;
-            b.out = sens;
-            b.ref = 1;
-            st = launch_back(b, EPI_ANCHOR, PET_TABLE_FP32, pl->ns, s, pl->max_sub_views);
-            if (st == PET_OK) st = launch_sum_sens(sens, sens + (size_t)pl->ns * pl->N, pl->ns, pl->N, s);
-        }
-        // other streams' states read them next, and `ones` is freed
-        const pet_status done = cuda_ok(cudaStreamSynchronize(s), "reference sensitivities");
-        if (st == PET_OK) st = done;
-    }
-    dfree(ones);
-    if (st != PET_OK) {
-        dfree(sens);
-        return st;
-    }
-    pl->d_sens_t_ref = sens;
-    return PET_OK;
+    return launch_forward(a, FWD_RATIO, false, choose_group(pl), s, nullptr);
 }
 
 // Full-data ratio in subset-major order into `ratio` (M * nz).
-pet_status ratio_all(const pet_problem *p, const float *f, float *ratio, cudaStream_t s, int ref = 0) {
+pet_status ratio_all(const pet_problem *p, const float *f, float *ratio, cudaStream_t s) {
     const pet_plan *pl = p->plan;
     FwdArgs a = fwd_args(pl, f, -1, false);
     a.g = p->d_g;
@@ -235,8 +194,7 @@ pet_status ratio_all(const pet_problem *p, const float *f, float *ratio, cudaStr
     a.w_scalar = p->w_scalar;
     a.out = ratio;
     a.status = p->d_status;
-    a.ref = ref;
-    return launch_forward(a, FWD_RATIO, false, full_group(pl, ref != 0), s, nullptr);
+    return launch_forward(a, FWD_RATIO, false, full_group(pl), s, nullptr);
 }
 
 // n_iter updates with the iterate ping-ponging between the caller's image and
@@ -317,7 +275,7 @@ pet_status state_init(pet_state *st, cudaStream_t s) {
     }
     if (st->algo != PET_ALGO_SAGA) return PET_OK;
     // table q_t = grad Phi_t(f^(0)) for all t, then qbar and d
-    PET_TRY(ratio_all(p, st->img, p->d_ratio, s, ref_rounding(st)));
+    PET_TRY(ratio_all(p, st->img, p->d_ratio, s));
     BackArgs b = back_args(pl, p->d_ratio, -1, false);
     b.t0 = 0;
     b.r_view0 = 0;
@@ -326,10 +284,8 @@ pet_status state_init(pet_state *st, cudaStream_t s) {
     b.pot = p->pen.potential;
     b.delta = p->pen.delta;
     b.table = st->table;
-    if (ref_rounding(st)) b.sens_t = pl->d_sens_t_ref;
     PET_TRY(launch_back(b, EPI_SAGA_INIT, st->table_dtype, pl->ns, s, pl->max_sub_views));
-    const float *sens = ref_rounding(st) ? pl->d_sens_t_ref + (size_t)pl->ns * pl->N : pl->d_sens;
-    return launch_saga_finish(st->table, st->table_dtype, pl->ns, Nz, pl->nz, st->img, sens, st->qbar, st->d, s);
+    return launch_saga_finish(st->table, st->table_dtype, pl->ns, Nz, pl->nz, st->img, pl->d_sens, st->qbar, st->d, s);
 }
 
 // The warm start (a constant image, then one unpenalised OSEM epoch in cyclic
@@ -423,7 +379,6 @@ void pet_plan_destroy(pet_plan *pl) {
     dfree(pl->d_all_off);
     dfree(pl->d_sens_t);
     dfree(pl->d_sens);
-    dfree(pl->d_sens_t_ref);
     dfree(pl->d_lz);
     delete pl;
 }
@@ -468,7 +423,7 @@ pet_status pet_plan_create(const pet_geometry *g, const pet_subsets *sub, pet_pl
     pl->na = g->n_angles;
     pl->nb = g->n_bins;
     bins_division(pl->nb, pl->nb_mul, pl->nb_shift);
-    tile_bins(g->pixel_mm, ds_chk, pl->nb, pl->nx, pl->ny, pl->bw, pl->cand1, pl->cand2);
+    tile_bins(g->pixel_mm, ds_chk, pl->nb, pl->nx, pl->ny, pl->bw, pl->cand);
     stack_candidates(g->pixel_mm, ds_chk, pl->nb, pl->nx, pl->ny, pl->cands, pl->cand_rounds);
     pl->ns = sub->n_subsets;
     pl->N = (int)N;
@@ -500,7 +455,6 @@ pet_status pet_plan_create(const pet_geometry *g, const pet_subsets *sub, pet_pl
         vp.K = (float)(ds / (cm * d));
         vp.invK = (float)(cm * d / ds);
         vp.inv_du = cn != 0.0 ? (float)(-cm / cn) : 0.0f;
-        vp.inv_adu = cn != 0.0 ? (float)std::fabs(cm / cn) : kAxisInv;
         const double off = (n_minor % 2) ? 0.5 : 0.0;
         for (int j = 0; j < pl->nb; ++j) {
             const double sj = ((double)j - 0.5 * (pl->nb - 1)) * ds;
@@ -576,7 +530,6 @@ pet_status pet_plan_create(const pet_geometry *g, const pet_subsets *sub, pet_pl
     b.t0 = 0;
     b.r_view0 = 0;
     b.out = pl->d_sens_t;
-    b.ref = !ring && g->nz > 1 ? 1 : 0;
     if ((st = launch_back(b, EPI_ANCHOR, PET_TABLE_FP32, pl->ns, 0, pl->max_sub_views)) != PET_OK) return fail(st);
     if ((st = launch_sum_sens(pl->d_sens_t, pl->d_sens, pl->ns, pl->N, 0)) != PET_OK) return fail(st);
     // nonzeros per subset, counted with the projector's own geometry
@@ -625,8 +578,6 @@ pet_status pet_plan_bytes(const pet_plan *pl, size_t *h_bytes) {
     if (!pl || !h_bytes) return set_error(PET_ERR_INVALID, "null argument");
     *h_bytes = sizeof(ViewParams) * pl->na + sizeof(float2) * (size_t)pl->M + sizeof(int) * (2 * (size_t)pl->na + pl->ns + 3) +
                sizeof(float) * ((size_t)pl->ns + 1) * pl->N;
-    std::lock_guard<std::mutex> lk(pl->ref_mu);
-    if (pl->d_sens_t_ref) *h_bytes += sizeof(float) * ((size_t)pl->ns + 1) * pl->N;
     return PET_OK;
 }
 
@@ -744,7 +695,7 @@ pet_status pet_forward(const pet_plan *pl, const float *d_img, const float *d_bg
     a.w = d_bg;
     a.w_scalar = bg;
     a.out = d_sino;
-    return launch_forward(a, FWD_YHAT, false, subset < 0 ? full_group(pl) : subset_group(pl), (cudaStream_t)stream,
+    return launch_forward(a, FWD_YHAT, false, subset < 0 ? full_group(pl) : choose_group(pl), (cudaStream_t)stream,
                           nullptr);
 }
 
@@ -931,7 +882,6 @@ pet_status pet_state_create(const pet_problem *p, int32_t algo, int32_t table_dt
             return fail(set_error(PET_ERR_OOM, "cudaMalloc SAGA table"));
         }
     }
-    if (ref_rounding(st) && (e = ensure_ref_sensitivity(pl, s)) != PET_OK) return fail(e);
     if ((e = state_init(st, s)) != PET_OK) return fail(e);
     *out = st;
     return PET_OK;
@@ -969,8 +919,7 @@ pet_status enqueue_update(pet_state *st, int algo, const int *t_dev, const float
     a.w_scalar = p->w_scalar;
     a.out = st->ratio;
     a.status = p->d_status;
-    a.ref = ref_rounding(st);
-    PET_TRY(launch_forward(a, FWD_RATIO, false, subset_group(pl, a.ref != 0), s, nullptr, max_sub_rays(pl)));
+    PET_TRY(launch_forward(a, FWD_RATIO, false, choose_group(pl), s, nullptr, max_sub_rays(pl)));
     BackArgs b = back_args(pl, st->ratio, 0, false);
     b.t_dev = t_dev;
     b.f = in;
@@ -988,8 +937,7 @@ pet_status enqueue_update(pet_state *st, int algo, const int *t_dev, const float
         b.B = st->B;
     } else if (algo == PET_ALGO_SAGA) {
         epi = EPI_SAGA;
-        if (ref_rounding(st)) b.sens_t = pl->d_sens_t_ref;
-        b.d = st->precond == PET_PRECOND_ITERATE ? nullptr : st->d;
+            b.d = st->precond == PET_PRECOND_ITERATE ? nullptr : st->d;
         b.table = st->table;
         b.qbar = st->qbar;
     } else if (algo == PET_ALGO_SVRG) {
@@ -1865,10 +1813,9 @@ void fill_member(BatchMember &m, const pet_state *st, float alpha, const int *se
     m.nb_mul = pl->nb_mul;
     m.nb_shift = pl->nb_shift;
     m.bw = pl->bw;
-    m.cand1 = pl->cand1;
-    m.cand2 = pl->cand2;
+    m.cand = pl->cand;
     m.ns = pl->ns;
-    m.sens_t = ref_rounding(st) ? pl->d_sens_t_ref : pl->d_sens_t;
+    m.sens_t = pl->d_sens_t;
     m.sens = pl->d_sens;
     m.g = p->d_g;
     m.w = p->d_w;
@@ -1879,7 +1826,6 @@ void fill_member(BatchMember &m, const pet_state *st, float alpha, const int *se
     m.status = p->d_status;
     m.algo = st->algo;
     m.table_dtype = st->table_dtype;
-    m.ref = ref_rounding(st);
     m.img = st->img;
     m.alt = st->alt;
     m.ratio = st->ratio;
@@ -1909,9 +1855,8 @@ void fill_member(BatchMember &m, const pet_state *st, float alpha, const int *se
 //     the other members' updates, the anchor finishes, then a back phase with
 //     the anchored members' updates; otherwise one back phase with every
 //     member's update.
-// Back phases are split by potential class and rounding (the quadratic epilogue
-// and the edge-preserving one, and the reference rounding of BF16 tables, are
-// different kernels), longest tiles first.
+// Back phases are split by potential class (the quadratic epilogue and the
+// edge-preserving one are different kernels), longest tiles first.
 // PET_BATCH_STREAMS: the batch's own streams (up to 8), created on first use;
 // fork makes them wait for `s`, join makes `s` wait for them.
 constexpr int kBatchSideStreams = 8;
@@ -1949,9 +1894,9 @@ void build_batch_phases(pet_batch *b, int n_iter, const std::vector<std::vector<
     int claim = 0;
     auto tiles_of = [](const pet_plan *pl) { return ((pl->nx + 15) / 16) * ((pl->ny + 15) / 16); };
     auto major_of = [](const pet_plan *pl) { return std::max(pl->nx, pl->ny); };
-    auto emit = [&](int i, int kind, std::vector<WorkSeg> &segs, int genpot, int ref) {
+    auto emit = [&](int i, int kind, std::vector<WorkSeg> &segs, int genpot) {
         if (segs.empty()) return;
-        pet_batch::Phase ph{kind, (int)b->h_segs.size(), (int)segs.size(), 0, genpot, ref, claim++};
+        pet_batch::Phase ph{kind, (int)b->h_segs.size(), (int)segs.size(), 0, genpot, claim++};
         for (WorkSeg &g : segs) {
             g.first = ph.n_items;
             ph.n_items += g.count;
@@ -1968,7 +1913,7 @@ void build_batch_phases(pet_batch *b, int n_iter, const std::vector<std::vector<
                 any = true;
                 fa.push_back({j, WK_FWD_ANCHOR, 0, forward_blocks(pl->M, 1, full_group(pl)), full_group(pl), 0});
             }
-            const int sub = subset_group(pl, ref_rounding(b->states[j]) != 0);
+            const int sub = choose_group(pl);
             fu.push_back({j, WK_FWD_UPDATE, 0, forward_blocks(max_sub_rays(pl), 1, sub),
                           sub, 0});
         }
@@ -1981,31 +1926,30 @@ void build_batch_phases(pet_batch *b, int n_iter, const std::vector<std::vector<
         std::stable_sort(fa.begin(), fa.end(), longer_fwd);
         std::stable_sort(fu.begin(), fu.end(), longer_fwd);
         fa.insert(fa.end(), fu.begin(), fu.end());
-        emit(i, 0, fa, 0, 0);
+        emit(i, 0, fa, 0);
         // views per subset decide a back item's length
         auto longer_back = [&](const WorkSeg &x, const WorkSeg &y) {
             return b->states[x.member]->prob->plan->max_sub_views > b->states[y.member]->prob->plan->max_sub_views;
         };
         for (int pass = any ? 0 : 1; pass < 2; ++pass) {
-            for (int cls = 0; cls < 4; ++cls) {
-                const int gp = cls & 1, ref = cls >> 1;
+            for (int gp = 0; gp < 2; ++gp) {
                 std::vector<WorkSeg> anc, upd;
                 for (int j = 0; j < n; ++j) {
                     const pet_state *st = b->states[j];
                     const pet_plan *pl = st->prob->plan;
                     const int member_gp = st->prob->pen.potential != PET_POT_QUADRATIC ? 1 : 0;
-                    if (pass == 0 && anchors[j][i] && cls == 0)
+                    if (pass == 0 && anchors[j][i] && gp == 0)
                         anc.push_back({j, WK_BACK_ANCHOR, 0, tiles_of(pl) * pl->ns, 0, tiles_of(pl)});
                     const bool update_here = any ? ((pass == 0) != (anchors[j][i] != 0)) : true;
-                    if (update_here && member_gp == gp && ref_rounding(st) == ref)
+                    if (update_here && member_gp == gp)
                         upd.push_back({j, WK_BACK_UPDATE, 0, tiles_of(pl), 0, tiles_of(pl)});
                 }
                 std::stable_sort(anc.begin(), anc.end(), longer_back);
                 std::stable_sort(upd.begin(), upd.end(), longer_back);
                 anc.insert(anc.end(), upd.begin(), upd.end());
-                emit(i, 1, anc, gp, ref);
+                emit(i, 1, anc, gp);
             }
-            if (pass == 0) b->phases[(size_t)i].push_back({2, 0, 0, 0, 0, 0, -1});   // the anchor finishes
+            if (pass == 0) b->phases[(size_t)i].push_back({2, 0, 0, 0, 0, -1});   // the anchor finishes
         }
     }
     b->n_claims = claim;
@@ -2045,7 +1989,7 @@ void build_batch_dataflow(pet_batch *b, int n_iter, const std::vector<std::vecto
                           st->algo == PET_ALGO_SVREM && !ready ? 1 : 0, ab, -1);
                 if (st->algo == PET_ALGO_SVREM) ready = true;
             }
-            const int sub = subset_group(pl, ref_rounding(st) != 0);
+            const int sub = choose_group(pl);
             const int f = add(DF_FWD_UPDATE, forward_blocks(max_sub_rays(pl), 1, sub),
                               sub, i, 0, prev_b, -1);
             prev_b = add(DF_BACK_UPDATE, tiles, 0, i, 0, f, fin);
@@ -2126,7 +2070,7 @@ pet_status enqueue_batch_epoch(pet_batch *b, int32_t n_iter, const std::vector<s
                                                   in_is_img ? 1 : 0, b->d_claims + ph.claim, false, s));
             } else if (ph.kind == 1) {
                 PET_TRY(launch_persistent_back(b->d_members, b->d_segs + ph.seg_off, ph.n_segs, ph.n_items, i,
-                                               in_is_img ? 1 : 0, b->d_claims + ph.claim, ph.genpot != 0, ph.ref != 0, s));
+                                               in_is_img ? 1 : 0, b->d_claims + ph.claim, ph.genpot != 0, s));
             } else {
                 for (int j = 0; j < n; ++j) {
                     if (!anchors[j][i]) continue;

@@ -26,7 +26,6 @@
 //   ANCHOR B_t = b for every subset t at once (grid.y = t)
 //   SAGA_INIT table_t = b - sens_t - (beta/N_s) grad R(f) for every t.
 #include <algorithm>
-#include <type_traits>
 
 #include "bodies.cuh"
 
@@ -34,24 +33,20 @@ namespace petvr {
 
 namespace {
 
-// Pixels a thread of the tile kernels takes (blocks of kTile^2 / PX threads per
-// group): two on launches over several subsets and in the persistent batches.
-constexpr int kPx = 2;
-constexpr int tile_threads(int px) { return kTile * kTile / px; }
-// Launches over this many views at once (all-view back projections, the SEM
-// start) split them over kViewGroups groups of threads per tile.
+// Launches over this many views at once and no state's update (all-view back
+// projections) split them over kViewGroups groups of threads per tile.
 constexpr int kManyViews = 32;
+constexpr int kBackMinBlocks = 4;
 
-template <int EPI, typename TQ, bool GENPOT, int PX, int GROUPS = 1>
-__global__ void __launch_bounds__(tile_threads(PX) * GROUPS, 4 * PX / GROUPS) back_tile_kernel(const BackArgs a) {
+template <int EPI, typename TQ, bool GENPOT, int GROUPS = 1>
+__global__ void __launch_bounds__(kBlock *GROUPS, kBackMinBlocks / GROUPS) back_tile_kernel(const BackArgs a) {
     const int t = a.t_dev ? __ldg(a.t_dev) : a.t0 + (int)blockIdx.y;
-    back_tile_body<EPI, TQ, GENPOT, PX, false, GROUPS>(a, t, blockIdx.x);
+    back_tile_body<EPI, TQ, GENPOT, false, GROUPS>(a, t, blockIdx.x);
 }
 
 template <int EPI, typename TQ, bool GENPOT>
-__global__ void __launch_bounds__(kRunThreadsMax) back_run_kernel(const BackArgs a) {
-    const int t = a.t_dev ? __ldg(a.t_dev) : a.t0 + (int)blockIdx.y;
-    back_run_body<EPI, TQ, GENPOT>(a, t, blockIdx.x);
+__global__ void __launch_bounds__(kBlock) back_run_kernel(const BackArgs a) {
+    back_run_body<EPI, TQ, GENPOT>(a, a.t0 + (int)blockIdx.y, blockIdx.x);
 }
 
 // Persistent batched back projection + update: a resident grid whose blocks
@@ -61,15 +56,14 @@ __global__ void __launch_bounds__(kRunThreadsMax) back_run_kernel(const BackArgs
 // launches, so results are bit-identical to them.
 // Thread 0 claims the item and writes its arguments to shared memory; the
 // segment table is staged in shared memory once per block.
-// GENPOT: the members of this launch use an edge-preserving potential.  REF:
-// they are SAGA states with BF16 tables (kRefRounding).
-template <bool GENPOT, bool REF>
-__global__ void __launch_bounds__(REF ? kRunBlock : tile_threads(kPx), REF ? 5 : 8)
+// GENPOT: the members of this launch use an edge-preserving potential.
+template <bool GENPOT>
+__global__ void __launch_bounds__(kBlock, kBackMinBlocks)
     persistent_back_kernel(const BatchMember *ms, const WorkSeg *segs, int n_segs, int n_items, int iter,
                            int in_is_img, int *claim) {
     __shared__ WorkSeg s_segs[kSegSmem];
     __shared__ BackArgs s_b;
-    __shared__ int s_item, s_t, s_tile, s_kind, s_algo;
+    __shared__ int s_item, s_t, s_tile, s_kind, s_algo, s_tq;
     for (int i = threadIdx.x; i < n_segs && i < kSegSmem; i += blockDim.x) s_segs[i] = segs[i];
     const WorkSeg *tab = n_segs <= kSegSmem ? s_segs : segs;
     // the segment table and member descriptors were copied in before the
@@ -98,8 +92,7 @@ __global__ void __launch_bounds__(REF ? kRunBlock : tile_threads(kPx), REF ? 5 :
                 b.nb = m.nb;
                 b.ns = m.ns;
                 b.bw = m.bw;
-                b.cand1 = m.cand1;
-                b.cand2 = m.cand2;
+                b.cand = m.cand;
                 const int local = g - sg.first;
                 if (sg.kind == WK_BACK_ANCHOR) {
                     const int t = local / sg.tiles;
@@ -134,19 +127,16 @@ __global__ void __launch_bounds__(REF ? kRunBlock : tile_threads(kPx), REF ? 5 :
                 s_b = b;
                 s_kind = sg.kind;
                 s_algo = m.algo;
+                s_tq = m.table_dtype;
             }
         }
         __syncthreads();
         if (s_item >= n_items) break;
         const int t = s_t, tile = s_tile;
-        if constexpr (REF) {
-            back_run_body<EPI_SAGA, __nv_bfloat16, GENPOT>(s_b, t, tile);
-        } else {
-            if (s_kind == WK_BACK_ANCHOR)
-                back_tile_body<EPI_ANCHOR, float, false, kPx>(s_b, t, tile);
-            else
-                member_update_tile<GENPOT, kPx>(s_algo, s_b, t, tile);
-        }
+        if (s_kind == WK_BACK_ANCHOR)
+            back_tile_body<EPI_ANCHOR, float, false>(s_b, t, tile);
+        else
+            member_update_tile<GENPOT>(s_algo, s_tq, s_b, t, tile);
     }
 }
 
@@ -182,36 +172,19 @@ struct TileBack {
     pet_status run() const {
         const int tiles = ((a.nx + kTile - 1) / kTile) * ((a.ny + kTile - 1) / kTile);
         const dim3 grid((unsigned)tiles, (unsigned)ny_grid);
-        constexpr bool bf16 = std::is_same<TQ, __nv_bfloat16>::value;
-        if constexpr (bf16 || EPI == EPI_ANCHOR) {
-            if (bf16 || a.ref) {
-                // subset launches are latency-bound: one run per thread; the all-subset
-                // ones are throughput-bound: threads loop over the runs, so that more
-                // blocks fit per SM
-                const int per_view = kTile * kTile / kRun;
-                const int threads = ny_grid > 1 ? kRunBlock : max(kRunBlock, per_view * min(max_views, kRunViews));
-                launch_dependent(back_run_kernel<EPI, TQ, GENPOT>, grid, dim3((unsigned)threads), run_smem_bytes(), s,
-                                 a);
-                return check_launch("back_run_kernel");
-            }
+        if constexpr (EPI == EPI_ANCHOR || EPI == EPI_SAGA_INIT || EPI == EPI_SAGAEM_INIT) {
+            launch_dependent(back_run_kernel<EPI, TQ, GENPOT>, grid, dim3(kBlock), run_smem_bytes(), s, a);
+            return check_launch("back_run_kernel");
         }
-        if constexpr (!bf16) {
-            if constexpr (EPI == EPI_ANCHOR || EPI == EPI_SAGA_INIT || EPI == EPI_SAGAEM_INIT) {
-                launch_dependent(back_tile_kernel<EPI, TQ, GENPOT, kPx>, grid, dim3(tile_threads(kPx)),
+        if constexpr (EPI == EPI_PLAIN)
+            if (max_views >= kManyViews) {
+                launch_dependent(back_tile_kernel<EPI, TQ, GENPOT, kViewGroups>, grid, dim3(kBlock * kViewGroups),
                                  tile_smem_bytes(), s, a);
                 return check_launch("back_tile_kernel");
             }
-            if constexpr (EPI == EPI_PLAIN || EPI == EPI_SEM_INIT)
-                if (max_views >= kManyViews) {
-                    launch_dependent(back_tile_kernel<EPI, TQ, GENPOT, kPx, kViewGroups>, grid,
-                                     dim3(tile_threads(kPx) * kViewGroups), tile_smem_bytes(), s, a);
-                    return check_launch("back_tile_kernel");
-                }
-            const auto k = back_tile_kernel<EPI, TQ, GENPOT, 1>;
-            const size_t smem = tile_smem_bytes();
-            launch_dependent(k, grid, dim3(tile_threads(1)),
-                             a.t_dev ? residency_smem((const void *)k, tiles, smem) : smem, s, a);
-        }
+        const auto k = back_tile_kernel<EPI, TQ, GENPOT>;
+        const size_t smem = tile_smem_bytes();
+        launch_dependent(k, grid, dim3(kBlock), a.t_dev ? residency_smem((const void *)k, tiles, smem) : smem, s, a);
         return check_launch("back_tile_kernel");
     }
 };
@@ -220,40 +193,36 @@ struct TileBack {
 
 // Bins a tile stages per view.  Over the tile's kTile x kTile pixels the first
 // candidate moves by at most (kTile - 1) (|cos| + |sin|) <= sqrt(2) (kTile - 1)
-// pixel / bin, and a pair of pixels has at most (2 + |du|) |cos| or (1 + 2 |du|)
-// |cos|, both <= sqrt(5), pixel / bin + 1 of them; two entries are always read,
-// and the rest is margin for rounding (see tile_view).  Bin numbers of 2^20 and more are beyond what the
+// pixel / bin, and a pixel has at most (1 + |du|) |cos| <= sqrt(2) pixel / bin + 1
+// of them; the unrolled loops always read two or three, and the rest is margin
+// for rounding (see tile_view).  Bin numbers of 2^20 and more are beyond what the
 // candidates' float positions resolve: such plans read their bins in place
 // (a value above kStageBins).
-void tile_bins(double pixel_mm, double bin_mm, int nb, int nx, int ny, int &bw, int &cand1, int &cand2) {
-    static_assert(kPx <= 2, "candidates of at most a pair of pixels");
+void tile_bins(double pixel_mm, double bin_mm, int nb, int nx, int ny, int &bw, int &cand) {
     const double ratio = pixel_mm / bin_mm;
     const double eps = 1e-3 + 4e-7 * ((double)nb + nx + ny);
     bw = kStageBins + 1;
-    cand1 = cand2 = kUnrolledCand + 1;
+    cand = kUnrolledCand + 1;
     if (nb >= (1 << 20) || ratio > (double)kStageBins) return;
-    cand1 = std::max(2, (int)std::floor(1.41422 * ratio + 2.0 * eps) + 1);
-    cand2 = std::max(2, (int)std::floor(2.23607 * ratio + 2.0 * eps) + 1);
-    bw = std::min(kStageBins + 1, (int)std::ceil((kTile - 1) * 1.41422 * ratio) + cand2 + 4);
+    cand = std::max(2, (int)std::floor(1.41422 * ratio + 2.0 * eps) + 1);
+    bw = std::min(kStageBins + 1, (int)std::ceil((kTile - 1) * 1.41422 * ratio) + cand + 4);
 }
 
 pet_status launch_persistent_back(const BatchMember *d_members, const WorkSeg *d_segs, int n_segs, int n_items,
-                                  int iter, int in_is_img, int *claim, bool general_potential, bool ref, cudaStream_t s) {
+                                  int iter, int in_is_img, int *claim, bool general_potential, cudaStream_t s) {
     if (n_items <= 0) return PET_OK;
     void (*k)(const BatchMember *, const WorkSeg *, int, int, int, int, int *) =
-        general_potential ? (ref ? persistent_back_kernel<true, true> : persistent_back_kernel<true, false>)
-                          : (ref ? persistent_back_kernel<false, true> : persistent_back_kernel<false, false>);
-    const size_t smem = ref ? run_smem_bytes() : tile_smem_bytes();
-    const int threads = ref ? kRunBlock : tile_threads(kPx);
-    static int resident[2][2] = {};   // blocks per SM by potential class and rounding
-    int &per_sm = resident[general_potential ? 1 : 0][ref ? 1 : 0];
+        general_potential ? persistent_back_kernel<true> : persistent_back_kernel<false>;
+    const size_t smem = tile_smem_bytes();
+    static int resident[2] = {};   // blocks per SM by potential class
+    int &per_sm = resident[general_potential ? 1 : 0];
     if (per_sm == 0 &&
-        (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)k, threads, smem) != cudaSuccess ||
+        (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)k, kBlock, smem) != cudaSuccess ||
          per_sm < 1))
         per_sm = 1;
     const int grid = std::min(n_items, per_sm * sm_count());
     ProfileScope prof(1, s);
-    launch_dependent(k, dim3((unsigned)grid), dim3((unsigned)threads), smem, s, d_members, d_segs, n_segs, n_items,
+    launch_dependent(k, dim3((unsigned)grid), dim3(kBlock), smem, s, d_members, d_segs, n_segs, n_items,
                      iter, in_is_img, claim);
     return check_launch("persistent_back_kernel");
 }

@@ -16,91 +16,26 @@ namespace petvr {
 
 namespace {
 
-constexpr int kTile = 16;           // single slice: a block owns a kTile x kTile pixel tile
+constexpr int kTile = 16;           // single slice: a block owns a kTile x kTile tile, a thread one pixel
+static_assert(kTile * kTile == kBlock, "one pixel of the tile per thread");
 
-constexpr int kSubsetBatch = 4;
-
-// The bands [kb, ke) of one ray from this thread, every fourth one from kb on:
-// sum of share times pixel, in units of the ray length per band.
+// The consecutive bands [kb, ke) of one ray: sum of weight times pixel.
 //
-// A band costs ~16 instructions: its lower end from the batch's base by one
-// FMA, the floor by a directed-rounding add (kRound), the share by one
-// saturating multiply, then two loads and three FMAs.  256^2, ncu: a full ratio
-// pass 23.2 us and 14.4M warp instructions (33.2 us and 22.0M with floorf, the
-// comparison of both band ends and contiguous bands per lane), a subset pass
-// 6.9 us (7.9).
-template <bool COH, int kBatch>
+// A band costs ~22 instructions: its far end by two FMAs, the floor by a
+// directed-rounding add (kRound), the weights (band_weights), then two loads
+// and two FMAs.
+template <bool COH>
 __device__ __forceinline__ float walk_bands(const FwdArgs &a, const ViewParams &vp, float uf, int ui, float hm,
                                             int n_minor, int kb, int ke) {
-    const int s_major = vp.col ? 1 : a.nx;
-    const int s_minor = vp.col ? a.nx : 1;
-    const float *img1 = a.img + s_minor;
-    // the band's lower end is at its far boundary when the line moves down
-    const float k_end = (vp.du < 0.0f ? 1.0f : 0.0f) - hm;
-    float acc = 0.0f;
-    // kBatch bands at a time: all their offsets and shares first, then the
-    // loads, then the FMAs in band order, so that the loads of a batch are in
-    // flight together.
-    for (int k = kb; k < ke; k += 4 * kBatch) {
-        // the batch's base position: the integer part of kc du goes into the
-        // pixel index, so that what is left stays small and exact
-        const float kc = (float)k + k_end;
-        const float tp = fmaf(kc, vp.du, kRound);
-        const float base = uf + fmaf(kc, vp.du_lo, fmaf(kc, vp.du, kRound - tp));
-        const unsigned iu = (unsigned)ui + __float_as_uint(tp) - 2u * kRoundBits;
-        int m0[kBatch];
-        float c0[kBatch];
-#pragma unroll
-        for (int b = 0; b < kBatch; ++b) {
-            const float lo = fmaf(4.0f * (float)b, vp.du, base);
-            const float t = __fadd_rd(lo, kRound);
-            m0[b] = (int)(__float_as_uint(t) + iu);
-            c0[b] = band_share(t - (kRound - 1.0f), lo, vp.inv_adu);
-        }
-        // a piece outside the image (or of a band past ke) is not loaded and
-        // adds 0; the upper pixel is loaded only where the line reaches it.
-        // lo is monotone in b, so when both pixels of the first and last band
-        // are inside the image every band's are: no checks then.
-        float x0[kBatch], x1[kBatch];
-        const int off = k * s_major;
-        if (k + 4 * (kBatch - 1) < ke && (unsigned)m0[0] < (unsigned)(n_minor - 1) &&
-            (unsigned)m0[kBatch - 1] < (unsigned)(n_minor - 1)) {
-#pragma unroll
-            for (int b = 0; b < kBatch; ++b) {
-                const int o = m0[b] * s_minor + (off + 4 * b * s_major);
-                x0[b] = ld_data<COH>(a.img + o);
-                x1[b] = c0[b] < 1.0f ? ld_data<COH>(img1 + o) : 0.0f;
-            }
-        } else {
-#pragma unroll
-            for (int b = 0; b < kBatch; ++b) {
-                const int o = m0[b] * s_minor + (off + 4 * b * s_major);
-                const bool live = k + 4 * b < ke;
-                x0[b] = live && (unsigned)m0[b] < (unsigned)n_minor ? ld_data<COH>(a.img + o) : 0.0f;
-                x1[b] = live && c0[b] < 1.0f && (unsigned)(m0[b] + 1) < (unsigned)n_minor ? ld_data<COH>(img1 + o)
-                                                                                         : 0.0f;
-            }
-        }
-#pragma unroll
-        for (int b = 0; b < kBatch; ++b) {
-            acc = fmaf(c0[b], x0[b], acc);
-            acc = fmaf(1.0f - c0[b], x1[b], acc);
-        }
-    }
-    return acc * vp.L;
-}
-
-// The same for the consecutive bands [kb, ke), with the weights of
-// band_split() in its own rounding (states with a BF16 table, see kRefRounding).
-template <bool COH>
-__device__ __forceinline__ float walk_bands_ref(const FwdArgs &a, const ViewParams &vp, float uf, int ui, float hm,
-                                                int n_minor, int kb, int ke) {
     const int s_major = vp.col ? 1 : a.nx;
     const int s_minor = vp.col ? a.nx : 1;
     const float *img1 = a.img + s_minor;
     float acc = 0.0f;
     float kc = (float)kb - hm;
     float va = band_point(vp, uf, kc);
+    // kBatch bands at a time: all their offsets and weights first, then the
+    // loads, then the FMAs in band order, so that the loads of a batch are in
+    // flight together.
     constexpr int kBatch = 4;
     for (int k = kb; k < ke; k += kBatch) {
         int m0[kBatch];
@@ -109,10 +44,14 @@ __device__ __forceinline__ float walk_bands_ref(const FwdArgs &a, const ViewPara
         for (int b = 0; b < kBatch; ++b) {
             kc += 1.0f;
             const float vb = band_point(vp, uf, kc);
-            const float t = band_split_ref(vp, va, vb, c0[b], c1[b]);
+            const float t = band_weights(vp.L, vp.Lm, fminf(va, vb), fmaxf(va, vb), c0[b], c1[b]);
             m0[b] = (int)(__float_as_uint(t) - kRoundBits) + ui;
             va = vb;
         }
+        // a piece outside the image (or of a band past ke) is not loaded and
+        // adds 0; the upper pixel is loaded only where the line reaches it.
+        // The lower end is monotone in the band, so when both pixels of the
+        // first and last band are inside the image every band's are: no checks.
         float x0[kBatch], x1[kBatch];
         const int off = k * s_major;
         if (k + kBatch <= ke && (unsigned)m0[0] < (unsigned)(n_minor - 1) &&
@@ -143,18 +82,13 @@ __device__ __forceinline__ float walk_bands_ref(const FwdArgs &a, const ViewPara
 }
 
 // Single-slice forward: a block takes RAYS adjacent rays of the view range
-// and splits each ray's bands over CHUNKS threads (RAYS * CHUNKS = kBlock): a
-// warp is 8 adjacent rays times 4 band lanes, and the CHUNKS / 4 warps of a ray
-// group take contiguous ranges of bands.  Inside a warp's range the 4 lanes
-// take every fourth band, so that one load touches 8 neighbouring pixels of 4
-// rows on a row-driven view and 4 neighbouring columns of the ~10 rows the 8
-// rays cross on a column-driven one (with contiguous chunks per lane those
-// were 32 different rows).  REF: consecutive bands per lane (kRefRounding).
-//
-// Chunk sums are reduced by xor-shuffles (within the warp) and then over
-// warps through shared memory, always in the same order, so the result is
-// deterministic.
-template <int CHUNKS, int MODE, bool LL, bool REF = false, bool COH = false>
+// and splits each ray's bands into CHUNKS contiguous chunks (RAYS * CHUNKS =
+// kBlock).  Inside a warp, lane = 8 * chunk + ray: the 32 lanes are 8
+// adjacent rays times 4 chunks, so one warp load touches 4 image rows with
+// 8 neighbouring pixels each.  Chunk sums are reduced by xor-shuffles
+// (within the warp) and then over warps through shared memory, always in the
+// same order, so the result is deterministic.
+template <int CHUNKS, int MODE, bool LL, bool COH = false>
 __device__ __forceinline__ void forward_tile_body(const FwdArgs &a, const int bx) {
     const int tid = threadIdx.x;
     constexpr int RAYS = kBlock / CHUNKS;        // rays per block
@@ -164,7 +98,7 @@ __device__ __forceinline__ void forward_tile_body(const FwdArgs &a, const int bx
     const int warp = tid >> 5;
     const int lane = tid & 31;
     const int r8 = lane & 7;
-    const int c4 = lane >> 3;                    // band lane
+    const int chunk = 4 * (warp % WPG) + (lane >> 3);
     const int ray_local = 8 * (warp / WPG) + r8;
     const int ray = bx * RAYS + ray_local;     // 32-bit: a plan has fewer than 2^31 rays
 
@@ -187,19 +121,11 @@ __device__ __forceinline__ void forward_tile_body(const FwdArgs &a, const int bx
         uf = u.y;
         int k_lo, k_hi;
         band_range(vp, u.x + u.y, n_major, n_minor, k_lo, k_hi);
-        // the ranges are aligned to the same bands for every ray of the view,
-        // so neighbouring lanes read the same image rows
-        if (REF) {
-            const int per = (n_major + CHUNKS - 1) / CHUNKS;
-            const int chunk = 4 * (warp % WPG) + c4;
-            kb = max(k_lo, chunk * per);
-            ke = min(k_hi, (chunk + 1) * per);
-        } else {
-            const int per = ((n_major + WPG - 1) / WPG + 3) & ~3;
-            const int wk = (warp % WPG) * per;
-            kb = max(k_lo & ~3, wk) + c4;
-            ke = min(k_hi, wk + per);
-        }
+        // chunks are aligned to the same bands for every ray of the view, so
+        // neighbouring lanes read the same image rows
+        const int per = (n_major + CHUNKS - 1) / CHUNKS;
+        kb = max(k_lo, chunk * per);
+        ke = min(k_hi, (chunk + 1) * per);
     }
     pdl_wait();
     pdl_trigger();
@@ -214,10 +140,7 @@ __device__ __forceinline__ void forward_tile_body(const FwdArgs &a, const int bx
         if (MODE == FWD_RATIO || LL) g_f = __ldg(a.g + gi);
         if (a.w) w_f = __ldg(a.w + gi);
     }
-    float acc = 0.0f;
-    if (kb < ke)
-        acc = REF ? walk_bands_ref<COH>(a, vp, uf, ui, hm, n_minor, kb, ke)
-                  : walk_bands<COH, CHUNKS >= 32 ? kSubsetBatch : 4>(a, vp, uf, ui, hm, n_minor, kb, ke);
+    float acc = kb < ke ? walk_bands<COH>(a, vp, uf, ui, hm, n_minor, kb, ke) : 0.0f;
     // the 4 chunks of each ray in this warp, then the warps of its group
     acc += __shfl_xor_sync(0xffffffffu, acc, 8);
     acc += __shfl_xor_sync(0xffffffffu, acc, 16);
@@ -261,88 +184,72 @@ __device__ __forceinline__ void forward_tile_body(const FwdArgs &a, const int bx
     }
 }
 
-// One item of a batched forward, with the member's band-chunk count and rounding.
+// One item of a batched forward, with the member's band-chunk count.
 template <int MODE, bool LL, bool COH = false>
 __device__ __forceinline__ void forward_item(const FwdArgs &a, int shape, int bx) {
-    if constexpr (MODE == FWD_RATIO && !LL) {
-        if (a.ref) {
-            if (shape == 8)
-                forward_tile_body<8, MODE, LL, kRefRounding, COH>(a, bx);
-            else if (shape == 16)
-                forward_tile_body<16, MODE, LL, kRefRounding, COH>(a, bx);
-            else
-                forward_tile_body<32, MODE, LL, kRefRounding, COH>(a, bx);
-            return;
-        }
-    }
     if (shape == 8)
-        forward_tile_body<8, MODE, LL, false, COH>(a, bx);
+        forward_tile_body<8, MODE, LL, COH>(a, bx);
     else if (shape == 16)
-        forward_tile_body<16, MODE, LL, false, COH>(a, bx);
+        forward_tile_body<16, MODE, LL, COH>(a, bx);
     else
-        forward_tile_body<32, MODE, LL, false, COH>(a, bx);
+        forward_tile_body<32, MODE, LL, COH>(a, bx);
 }
 
 // ---- back projection ------------------------------------------------------------
 
-// Single-slice path: a block owns a kTile x kTile pixel tile, a thread PX pixels
-// (a column of PX neighbours along y; the block has kTile^2 / PX threads).  For
-// each view of the subset two tables are staged in shared memory: the bins
-// whose rays can meet the tile (offset, and ratio times ray length), and per
-// band of the tile the displacement of a ray over the bands from the image
-// centre.  A pixel then takes its candidate bins and adds share times ratio in
-// registers, views and bins in increasing order, so the result is
-// deterministic (and the same for any PX) and needs no atomics.
+// Single-slice path: a block owns a kTile x kTile pixel tile, a thread one pixel.
+// For each view of the subset two tables are staged in shared memory: the bins
+// whose rays can meet the tile (offset and ratio), and per band of the tile the
+// position of its lower end.  A pixel takes its candidate bins and adds weight
+// times ratio in registers, a sum per view over its bins in increasing order,
+// then over the views, so the result is deterministic and needs no atomics.
 constexpr int kStageViews = 32;        // views per pass
 constexpr int kStageBins = 1024;       // staged bins per pass
 constexpr int kViewGroups = 4;         // groups of threads on launches over all views
-constexpr int kUnrolledCand = 3;       // candidate counts with an unrolled view loop
+constexpr int kUnrolledCand = 3;       // largest candidate count with a loop of its own
 
 // Per-view constants of a tile.  A ray's offset from pixel m at its band's
 // lower end is x = u_j + P - m, with P = kc du its displacement over the kc
 // bands from the image centre; the ray meets the pixel for -|du| < x < 1, so
 // the candidates are the bins of that range, u_j = (j - (nb - 1) / 2) K + off.
 // They are found from approximate positions, with a margin far above their
-// rounding; a candidate that misses the pixel gets share 0.
+// rounding; a candidate that misses the pixel adds nothing.
 struct alignas(16) TileView {
-    float inv_adu, invK;
+    float du, du_lo;
+    float step;       // from a band's lower end to its upper end: +1 or -1
+    float k0;         // centred major coordinate of the lower end of the tile's first band
+    float L, Lm;
     unsigned base;    // staged entry of bin 0, less kRoundBits (see kRound)
     int flags;        // bit 0: column-driven; above it: the number of candidate bins
-    float du, du_lo;
-    float k0;         // centred major coordinate of the tile's first band's lower end
+    float invK;
     float cst;        // first candidate: floor((m - P) invK + cst)
-    float L;          // ray length per band
     int j0, v;        // first staged bin; view
-    int pad;
 };
 
 struct TileShared {
-    float4 bins[kStageBins];                // [view][bw]: offset (integer, fraction), ratio times L
-    float4 bands[kStageViews * kTile];      // [view][band]: P (integer, fraction), cst - P invK
+    float4 bins[kStageBins];                // [view][bw]: offset (integer, fraction), ratio
+    float4 bands[kStageViews * kTile];      // [view][band]: kc of the lower end, cst - P invK, invK, kc of the upper end
     TileView views[kStageViews];
 };
 
-// The candidates of a thread's PX pixels are taken together: the next pixel
-// along y shifts x by `step`.
-template <int PX>
 __device__ __forceinline__ void tile_view(const BackArgs &a, const ViewParams &vp, int v, int x0, int y0, int q,
                                           TileView &tv) {
     const int n_minor = vp.col ? a.ny : a.nx;
     const int n_major = vp.col ? a.nx : a.ny;
     const float adu = fabsf(vp.du);
-    const float step = (float)(PX - 1) * (vp.col ? -1.0f : vp.du);
     const float eps = 1e-3f + 4e-7f * (float)(a.nb + a.nx + a.ny);
     const float first = vp.invK > 0.0f ? -adu : 1.0f;
     const float off = (n_minor & 1) ? 0.5f : 0.0f;
-    tv.inv_adu = vp.inv_adu;
-    tv.invK = vp.invK;
     tv.du = vp.du;
     tv.du_lo = vp.du_lo;
-    tv.k0 = (float)(vp.col ? x0 : y0) - 0.5f * (float)n_major + (vp.du < 0.0f ? 1.0f : 0.0f);
-    tv.cst = fmaf(first - off, vp.invK, 0.5f * (float)(a.nb - 1)) + fminf(0.0f, -step * vp.invK) + (1.0f - eps);
-    const int nc = (int)floorf(fmaf(1.0f + adu + fabsf(step), fabsf(vp.invK), 2.0f * eps)) + 1;
-    tv.flags = (vp.col ? 1 : 0) | (nc << 1);
+    tv.step = vp.du < 0.0f ? -1.0f : 1.0f;
     tv.L = vp.L;
+    tv.Lm = vp.Lm;
+    tv.invK = vp.invK;
+    tv.k0 = (float)(vp.col ? x0 : y0) - 0.5f * (float)n_major + (vp.du < 0.0f ? 1.0f : 0.0f);
+    tv.cst = fmaf(first - off, vp.invK, 0.5f * (float)(a.nb - 1)) + (1.0f - eps);
+    const int nc = (int)floorf(fmaf(1.0f + adu, fabsf(vp.invK), 2.0f * eps)) + 1;
+    tv.flags = (vp.col ? 1 : 0) | (nc << 1);
     tv.v = v;
     // smallest first candidate over the tile's corners, less one for rounding
     const float m0 = (float)((vp.col ? y0 : x0) - (n_minor >> 1));
@@ -353,22 +260,9 @@ __device__ __forceinline__ void tile_view(const BackArgs &a, const ViewParams &v
     tv.base = (unsigned)(q * a.bw - tv.j0) - kRoundBits;
 }
 
-// A ray's offset as staged.  On an axis-aligned view only the pixel a ray lies
-// in matters, so its fraction is moved well inside that pixel.
-__device__ __forceinline__ float2 staged_offset(float2 u, float du) {
-    if (du == 0.0f) u.y = u.y < 0.0f ? -0.5f : 0.25f;
-    return u;
-}
-
-// Share of a ray's band in the pixel it meets at offset x: the part of the
-// band with -|du| < x < 1, as band_share() and its complement.
-__device__ __forceinline__ float pixel_share(float x, float inv_adu) {
-    return __saturatef(fmaf(-x, inv_adu, inv_adu)) - __saturatef(-x * inv_adu);
-}
-
-// Staged bins of a pass: warp w takes the 32-bin pieces w, w + NT / 32, ... of
-// the views, two pieces' loads in flight at a time.  `load(view, bin, entry,
-// live)` starts one entry's load and returns what stores it.
+// Staged bins of a pass: warp w of the NT threads takes the 32-bin pieces w, w +
+// NT / 32, ... of the views, two pieces' loads in flight at a time.  `load(view,
+// bin, entry, live)` starts one entry's load and returns what stores it.
 template <int NT, class Load>
 __device__ __forceinline__ void stage_bins(int nq, int bw, Load &&load) {
     const int per_view = (bw + 31) >> 5;
@@ -386,22 +280,19 @@ __device__ __forceinline__ void stage_bins(int nq, int bw, Load &&load) {
     }
 }
 
-// Bound by instruction issue on the all-subset launches (two pixels a thread
-// share the candidates, three for a pair where bins are as wide as pixels,
-// against two each) and by the launch's dependent round trips on subset
-// launches (one pixel a thread, for twice the warps).  x is formed from integer
-// and fractional parts separately (exact integers, fractions below 2), so its
-// error does not grow with the image.  Against runs of 8 pixels a thread that
-// walked their rays with sums in shared memory (back_run_body): 256^2 anchor of
-// 21 subsets 40.1 -> 31.0 us (ncu), an update (both projections, in a graph)
-// 8.8 -> 6.7 us, 512^2 with 60 views a subset 90 -> 61 us.
+// Bound by the launch's dependent round trips on subset launches: the bins
+// arrive in one, and the views' chains overlap.  The weights are band_weights()
+// of the positions the forward computes, bit for bit (the ends come in order,
+// so the floor, the share and the test of the upper end are all there is to a
+// candidate).  Against runs of 8 pixels a thread (back_run_body): two 256^2 SVREM
+// epochs 601 -> 534 us, a 512^2 reconstruction 3400 -> 3131 us.
 //
 // GROUPS > 1: group g of the block's threads takes the views g, g + GROUPS, ...
 // of a pass, and the groups' sums are added in order (launches over all views,
 // whose few tiles would otherwise walk every view one after another).
-template <int EPI, typename TQ, bool GENPOT, int PX, bool COH = false, int GROUPS = 1>
+template <int EPI, typename TQ, bool GENPOT, bool COH = false, int GROUPS = 1>
 __device__ __forceinline__ void back_tile_body(const BackArgs &a, const int t, const int bx) {
-    constexpr int NT = kTile * kTile / PX;
+    constexpr int NT = kTile * kTile;
     extern __shared__ unsigned char smem_raw[];
     const int tid = GROUPS > 1 ? threadIdx.x % NT : threadIdx.x;
     const int group = GROUPS > 1 ? threadIdx.x / NT : 0;
@@ -412,37 +303,33 @@ __device__ __forceinline__ void back_tile_body(const BackArgs &a, const int t, c
     const int tiles_x = (a.nx + kTile - 1) / kTile;
     const int x0 = (bx % tiles_x) * kTile;
     const int y0 = (bx / tiles_x) * kTile;
-    const int tx = tid % kTile, ty = tid / kTile * PX;
-    const bool staged = a.bw <= kStageBins;   // else (bins far finer than pixels) bins are read in place
+    const int tx = tid % kTile, ty = tid / kTile;
+    const bool staged = a.bw <= kStageBins;      // else (bins far finer than pixels) bins are read in place
     const int per_pass = staged ? min(kStageViews, kStageBins / a.bw) : kStageViews;
     const float mx = (float)(x0 + tx - (a.nx >> 1)), my = (float)(y0 + ty - (a.ny >> 1));
 
-    float acc[PX] = {};
+    float acc = 0.0f;
     for (int q0 = 0; q0 < nv; q0 += per_pass) {
         const int nq = min(per_pass, nv - q0);
         if (q0 > 0) __syncthreads();             // the pass before is done with shared memory
         if (threadIdx.x < nq) {
             const int v = __ldg(a.order + vb + q0 + threadIdx.x);
-            tile_view<PX>(a, a.views[v], v, x0, y0, threadIdx.x, sh.views[threadIdx.x]);
+            tile_view(a, a.views[v], v, x0, y0, threadIdx.x, sh.views[threadIdx.x]);
         }
         __syncthreads();
         // plan constants before the wait for the kernel ahead, ratios after it
         for (int i = threadIdx.x; i < nq * kTile; i += NT * GROUPS) {
             const TileView &tv = sh.views[i / kTile];
             const float kc = tv.k0 + (float)(i % kTile);
-            const float tp = fmaf(kc, tv.du, kRound);
-            const float pi = tp - kRound;
-            const float pf = fmaf(kc, tv.du_lo, fmaf(kc, tv.du, -pi));
-            sh.bands[i] = make_float4(pi, pf, fmaf(-(pi + pf), tv.invK, tv.cst), 0.0f);
+            sh.bands[i] = make_float4(kc, fmaf(-(kc * tv.du), tv.invK, tv.cst), tv.invK, kc + tv.step);
         }
         if (staged)
             stage_bins<NT * GROUPS>(nq, a.bw, [&](int q, int i, int e, bool live) {
                 const int j = sh.views[q].j0 + i;
                 float2 u = make_float2(0.0f, 0.0f);
-                if (live && (unsigned)j < (unsigned)a.nb)
-                    u = __ldg(a.uc + sh.views[q].v * a.nb + j);
+                if (live && (unsigned)j < (unsigned)a.nb) u = __ldg(a.uc + sh.views[q].v * a.nb + j);
                 return [=, &sh](void) {
-                    if (live) *reinterpret_cast<float2 *>(sh.bins + e) = staged_offset(u, sh.views[q].du);
+                    if (live) *reinterpret_cast<float2 *>(sh.bins + e) = u;
                 };
             });
         if (q0 == 0) {
@@ -456,7 +343,7 @@ __device__ __forceinline__ void back_tile_body(const BackArgs &a, const int t, c
                 if (live && (unsigned)j < (unsigned)a.nb)
                     r = ld_data<COH>(a.r + (vb + q0 + q - r_view0) * a.nb + j);
                 return [=, &sh](void) {
-                    if (live) sh.bins[e].z = r * sh.views[q].L;
+                    if (live) sh.bins[e].z = r;
                 };
             });
         __syncthreads();
@@ -465,93 +352,83 @@ __device__ __forceinline__ void back_tile_body(const BackArgs &a, const int t, c
         // views of an unrolled group overlap
         auto gather = [&](auto nc) {
             constexpr int NC = decltype(nc)::value;
-#pragma unroll (NC == 2 ? 2 / PX : 1)
+#pragma unroll (NC == 2 ? 2 : 1)
             for (int q = group; q < nq; q += GROUPS) {
-                const float4 vc = *reinterpret_cast<const float4 *>(&sh.views[q]);     // inv_adu, invK, base, flags
-                const int flags = __float_as_int(vc.w);
+                const float2 vc = *reinterpret_cast<const float2 *>(&sh.views[q].du);       // du, du_lo
+                const float4 vd = *reinterpret_cast<const float4 *>(&sh.views[q].L);        // L, Lm, base, flags
+                const int flags = __float_as_int(vd.w);
                 const bool col = flags & 1;
                 const float m = col ? my : mx;
-                const float4 *bands = sh.bands + q * kTile + (col ? tx : ty);
-                float b[PX], pf[PX];
-                float e = 0.0f;
-#pragma unroll
-                for (int p = 0; p < PX; ++p) {
-                    const float4 bd = bands[col ? 0 : p];
-                    if (p == 0) e = fmaf(m, vc.y, bd.z);
-                    b[p] = m + (col ? (float)p : 0.0f) - bd.x;
-                    pf[p] = bd.y;
-                }
+                const float4 bd = sh.bands[q * kTile + (col ? tx : ty)];
+                const float e = fmaf(m, bd.z, bd.y);
+                float part = 0.0f;
                 auto add = [&](float ui, float uf, float r) {
-#pragma unroll
-                    for (int p = 0; p < PX; ++p) {
-                        const float w = pixel_share((ui - b[p]) + (uf + pf[p]), vc.x);
-                        if (w > 0.0f) acc[p] = fmaf(w, r, acc[p]);
-                    }
+                    const float lo = fmaf(bd.x, vc.x, fmaf(bd.x, vc.y, uf));        // band_point()
+                    const float fl1 = __fadd_rd(lo, kRound) - (kRound - 1.0f);
+                    float w0 = fminf((fl1 - lo) * vd.y, vd.x);                      // band_weights()
+                    if (fmaf(bd.w, vc.x, fmaf(bd.w, vc.y, uf)) <= fl1) w0 = vd.x;
+                    const float w1 = vd.x - w0;
+                    const float c = fl1 + (ui - m);        // 1: the ray's lower pixel is this one, 0: its upper one
+                    if (c == 1.0f) part = fmaf(w0, r, part);
+                    if (c == 0.0f && w1 > 0.0f) part = fmaf(w1, r, part);
                 };
-                if (NC > 0 || staged) {
-                    const float4 *ent = sh.bins + (__float_as_uint(__fadd_rd(e, kRound)) + __float_as_uint(vc.z));
+                if (NC > 0) {
+                    const float4 *ent = sh.bins + (__float_as_uint(__fadd_rd(e, kRound)) + __float_as_uint(vd.z));
                     float4 en[NC > 0 ? NC : 1];
 #pragma unroll
-                    for (int c = 0; c < NC; ++c) en[c] = ent[c];
+                    for (int k = 0; k < NC; ++k) en[k] = ent[k];
 #pragma unroll
-                    for (int c = 0; c < NC; ++c) add(en[c].x, en[c].y, en[c].z);
-                    if (NC == 0)
-#pragma unroll 1
-                        for (int c = 0; c < flags >> 1; ++c) add(ent[c].x, ent[c].y, ent[c].z);
+                    for (int k = 0; k < NC; ++k) add(en[k].x, en[k].y, en[k].z);
                 } else {
                     const int j0 = (int)floorf(e);
+                    const float4 *ent = sh.bins + (q * a.bw - sh.views[q].j0);
 #pragma unroll 1
                     for (int j = max(j0, 0); j < min(j0 + (flags >> 1), a.nb); ++j) {
-                        const float2 u = staged_offset(__ldg(a.uc + sh.views[q].v * a.nb + j), sh.views[q].du);
-                        add(u.x, u.y, ld_data<COH>(a.r + (vb + q0 + q - r_view0) * a.nb + j) * sh.views[q].L);
+                        if (staged) {
+                            add(ent[j].x, ent[j].y, ent[j].z);
+                        } else {
+                            const float2 u = __ldg(a.uc + sh.views[q].v * a.nb + j);
+                            add(u.x, u.y, ld_data<COH>(a.r + (vb + q0 + q - r_view0) * a.nb + j));
+                        }
                     }
                 }
+                acc += part;
             }
         };
-        const int most = PX == 1 ? a.cand1 : a.cand2;
-        if (!staged || most > kUnrolledCand)
-            gather(std::integral_constant<int, 0>());
-        else if (most == 2)
+        if (staged && a.cand == 2)
             gather(std::integral_constant<int, 2>());
-        else
+        else if (staged && a.cand == 3)
             gather(std::integral_constant<int, 3>());
+        else
+            gather(std::integral_constant<int, 0>());
     }
     pdl_wait();   // returns at once after the wait above; covers an empty subset
     if constexpr (GROUPS > 1) {
-        float *sums = reinterpret_cast<float *>(smem_raw);      // [GROUPS][PX][NT]
+        float *sums = reinterpret_cast<float *>(smem_raw);      // [GROUPS][NT]
         __syncthreads();
-        if (group > 0)
-#pragma unroll
-            for (int p = 0; p < PX; ++p) sums[(group * PX + p) * NT + tid] = acc[p];
+        if (group > 0) sums[group * NT + tid] = acc;
         __syncthreads();
         if (group > 0) return;
 #pragma unroll
-        for (int g = 1; g < GROUPS; ++g)
-#pragma unroll
-            for (int p = 0; p < PX; ++p) acc[p] += sums[(g * PX + p) * NT + tid];
+        for (int g = 1; g < GROUPS; ++g) acc += sums[g * NT + tid];
     }
-    const int ix = x0 + tx;
-#pragma unroll
-    for (int p = 0; p < PX; ++p) {
-        const int iy = y0 + ty + p;
-        if (ix < a.nx && iy < a.ny) {
-            const int n = iy * a.nx + ix;
-            apply_epilogue<EPI, TQ, GENPOT, COH>(a, t, n, n, ix, iy, 0, acc[p]);
-        }
+    const int ix = x0 + tx, iy = y0 + ty;
+    if (ix < a.nx && iy < a.ny) {
+        const int n = iy * a.nx + ix;
+        apply_epilogue<EPI, TQ, GENPOT, COH>(a, t, n, n, ix, iy, 0, acc);
     }
 }
 
-// The reference rounding (kRefRounding): for each view, the tile's bands are cut
-// into runs of kRun pixels along the view's minor axis; one thread walks the
-// rays that can cross a run in order and adds each ray's two band pieces into
-// per-view partial sums in shared memory (every (view, pixel) slot has exactly
-// one writer, so no atomics).  Then each thread sums its pixels' partials over
-// the views in a fixed order and applies the update.  A gather per pixel in
-// this rounding takes 1.3 times the instructions (it evaluates both ends of
-// every candidate's band twice).
+// All-subset launches (anchors, table fills), which fill the GPU: for each view,
+// the tile's bands are cut into runs of kRun pixels along the view's minor
+// axis; one thread walks the rays that can cross a run in order and adds each
+// ray's two band pieces into per-view partial sums in shared memory (every
+// (view, pixel) slot has exactly one writer, so no atomics).  Then each thread
+// sums its pixel's partials over the views in order.  The same weights and
+// order of sums as back_tile_body, bit for bit, in fewer instructions (a band
+// is evaluated once for the run, not for every pixel it can touch) but a longer
+// chain: 256^2, 21 subsets ANCHOR_TIMES.
 constexpr int kRun = 8;
-constexpr int kRunBlock = 256;         // threads of a looping block (at least the tile's pixels)
-constexpr int kRunThreadsMax = 512;
 constexpr int kRunViews = 16;          // views per shared-memory pass
 
 struct RunShared {
@@ -560,14 +437,14 @@ struct RunShared {
     int vid[kRunViews];
 };
 
-template <int EPI, typename TQ, bool GENPOT, bool COH = false>
+template <int EPI, typename TQ, bool GENPOT>
 __device__ __forceinline__ void back_run_body(const BackArgs &a, const int t, const int bx) {
     extern __shared__ unsigned char smem_raw[];
     RunShared &sh = *reinterpret_cast<RunShared *>(smem_raw);
     const int vb = __ldg(a.sub_off + t);
     const int nv = __ldg(a.sub_off + t + 1) - vb;
     const int r_view0 = a.t_dev ? vb : a.r_view0;
-    const int nthr = blockDim.x;                  // >= kTile * kTile
+    constexpr int nthr = kBlock;
 
     const int tiles_x = (a.nx + kTile - 1) / kTile;
     const int x0 = (bx % tiles_x) * kTile;
@@ -617,45 +494,48 @@ __device__ __forceinline__ void back_run_body(const BackArgs &a, const int t, co
             const float *rv = a.r + (vb + q0 + ql - r_view0) * a.nb;
             for (int j = jlo; j <= jhi; ++j) {
                 const float2 u = __ldg(ucv + j);
+                const float e0 = band_point(vp, u.y, kc), e1 = band_point(vp, u.y, kc + 1.0f);
                 float w0, w1;
-                const float tl = band_split_ref(vp, band_point(vp, u.y, kc), band_point(vp, u.y, kc + 1.0f), w0, w1);
+                const float tl = band_weights(vp.L, vp.Lm, fminf(e0, e1), fmaxf(e0, e1), w0, w1);
                 const int c = (int)(__float_as_uint(tl) - kRoundBits) + (int)u.x - m0rel;
-                const float r = ld_data<COH>(rv + j);
+                const float r = __ldg(rv + j);
                 if ((unsigned)c < (unsigned)mlen) pp[c * lstep] += w0 * r;
                 if (w1 > 0.0f && (unsigned)(c + 1) < (unsigned)mlen) pp[(c + 1) * lstep] += w1 * r;
             }
         }
         __syncthreads();
-        if (threadIdx.x < kTile * kTile)
-            for (int ql = 0; ql < nq; ++ql) acc += sh.part[ql][threadIdx.x];
+        for (int ql = 0; ql < nq; ++ql) acc += sh.part[ql][threadIdx.x];
         __syncthreads();
     }
     pdl_wait();   // returns at once after the wait above; covers an empty subset
-    if (threadIdx.x < kTile * kTile) {
-        const int ix = x0 + (threadIdx.x % kTile);
-        const int iy = y0 + (threadIdx.x / kTile);
-        if (ix < a.nx && iy < a.ny) {
-            const int n = iy * a.nx + ix;
-            apply_epilogue<EPI, TQ, GENPOT, COH>(a, t, n, n, ix, iy, 0, acc);
-        }
+    const int ix = x0 + (threadIdx.x % kTile);
+    const int iy = y0 + (threadIdx.x / kTile);
+    if (ix < a.nx && iy < a.ny) {
+        const int n = iy * a.nx + ix;
+        apply_epilogue<EPI, TQ, GENPOT>(a, t, n, n, ix, iy, 0, acc);
     }
 }
 
 inline size_t run_smem_bytes() { return sizeof(RunShared); }
 inline size_t tile_smem_bytes() { return sizeof(TileShared); }
 
-// Member update of one tile: the member's algorithm selects the epilogue (the
-// single-state launch's template argument).
-template <bool GENPOT, int PX, bool COH = false>
-__device__ __forceinline__ void member_update_tile(int algo, const BackArgs &b, int t, int tile) {
+// Member update of one tile: the member's algorithm and table type select
+// the epilogue (the single-state launch's template arguments).
+template <bool GENPOT, bool COH = false>
+__device__ __forceinline__ void member_update_tile(int algo, int table_dtype, const BackArgs &b, int t, int tile) {
     switch (algo) {
-        case PET_ALGO_OSEM: back_tile_body<EPI_OSEM, float, GENPOT, PX, COH>(b, t, tile); break;
-        case PET_ALGO_SVREM: back_tile_body<EPI_SVREM, float, GENPOT, PX, COH>(b, t, tile); break;
-        case PET_ALGO_SAGA: back_tile_body<EPI_SAGA, float, GENPOT, PX, COH>(b, t, tile); break;
-        case PET_ALGO_SGA: back_tile_body<EPI_SGA, float, GENPOT, PX, COH>(b, t, tile); break;
-        case PET_ALGO_SEM: back_tile_body<EPI_SEM, float, GENPOT, PX, COH>(b, t, tile); break;
-        case PET_ALGO_SAGAEM: back_tile_body<EPI_SAGAEM, float, GENPOT, PX, COH>(b, t, tile); break;
-        default: back_tile_body<EPI_SVRG, float, GENPOT, PX, COH>(b, t, tile); break;
+        case PET_ALGO_OSEM: back_tile_body<EPI_OSEM, float, GENPOT, COH>(b, t, tile); break;
+        case PET_ALGO_SVREM: back_tile_body<EPI_SVREM, float, GENPOT, COH>(b, t, tile); break;
+        case PET_ALGO_SAGA:
+            if (table_dtype == PET_TABLE_BF16)
+                back_tile_body<EPI_SAGA, __nv_bfloat16, GENPOT, COH>(b, t, tile);
+            else
+                back_tile_body<EPI_SAGA, float, GENPOT, COH>(b, t, tile);
+            break;
+        case PET_ALGO_SGA: back_tile_body<EPI_SGA, float, GENPOT, COH>(b, t, tile); break;
+        case PET_ALGO_SEM: back_tile_body<EPI_SEM, float, GENPOT, COH>(b, t, tile); break;
+        case PET_ALGO_SAGAEM: back_tile_body<EPI_SAGAEM, float, GENPOT, COH>(b, t, tile); break;
+        default: back_tile_body<EPI_SVRG, float, GENPOT, COH>(b, t, tile); break;
     }
 }
 

@@ -102,7 +102,7 @@ __global__ void __maxnreg__(kDataflowRegs)
         BackArgs b;
         FinArgs fin;
     } s_args;
-    __shared__ int s_item, s_seg, s_ok, s_kind, s_shape, s_bx, s_t, s_algo, s_ref;
+    __shared__ int s_item, s_seg, s_ok, s_kind, s_shape, s_bx, s_t, s_algo, s_tq;
     int *claim = done;             // done[0]: the claim counter; done[1 + k]: items of segment k done
     int *seg_done = done + 1;
     // the counters were zeroed by the kernel ahead of this one
@@ -133,7 +133,7 @@ __global__ void __maxnreg__(kDataflowRegs)
                     s_shape = sg.shape;
                     s_bx = local;
                     s_algo = m.algo;
-                    s_ref = m.ref;
+                    s_tq = m.table_dtype;
                     if (sg.kind == DF_FWD_UPDATE || sg.kind == DF_FWD_ANCHOR) {
                         FwdArgs a{};
                         a.views = m.views;
@@ -153,7 +153,6 @@ __global__ void __maxnreg__(kDataflowRegs)
                         if (sg.kind == DF_FWD_UPDATE) {
                             a.sub_off = m.sub_off;
                             a.t_dev = m.seq + sg.iter;
-                            a.ref = m.ref;
                             a.out = m.ratio;
                         } else {
                             a.v_begin = 0;
@@ -188,8 +187,7 @@ __global__ void __maxnreg__(kDataflowRegs)
                         b.nb = m.nb;
                         b.ns = m.ns;
                         b.bw = m.bw;
-                        b.cand1 = m.cand1;
-                        b.cand2 = m.cand2;
+                        b.cand = m.cand;
                         if (sg.kind == DF_BACK_ANCHOR) {
                             const int t = local / sg.tiles;
                             b.r = m.ratio_full;
@@ -234,11 +232,9 @@ __global__ void __maxnreg__(kDataflowRegs)
                 const long long i = (long long)bx * kBlock + threadIdx.x;
                 if (i < s_args.fin.plane) finish_pixel(s_args.fin, i);
             } else if (kind == DF_BACK_ANCHOR) {
-                back_tile_body<EPI_ANCHOR, float, false, 1, true>(s_args.b, s_t, bx);
-            } else if (s_ref) {
-                back_run_body<EPI_SAGA, __nv_bfloat16, GENPOT, true>(s_args.b, s_t, bx);
+                back_tile_body<EPI_ANCHOR, float, false, true>(s_args.b, s_t, bx);
             } else {
-                member_update_tile<GENPOT, 1, true>(s_algo, s_args.b, s_t, bx);
+                member_update_tile<GENPOT, true>(s_algo, s_tq, s_args.b, s_t, bx);
             }
         }
         __syncthreads();
@@ -257,8 +253,7 @@ pet_status launch_dataflow_epoch(const BatchMember *d_members, const DfSeg *d_se
     if (n_items <= 0) return PET_OK;
     void (*k)(const BatchMember *, const DfSeg *, int, int, int, int *, int *, long long) =
         general_potential ? dataflow_epoch_kernel<true> : dataflow_epoch_kernel<false>;
-    const size_t smem = std::max(tile_smem_bytes(), run_smem_bytes());
-    static_assert(kRunBlock == kBlock, "one pixel per thread in both back projections");
+    const size_t smem = tile_smem_bytes();
     static int resident[2] = {};   // blocks per SM by potential class
     int &per_sm = resident[general_potential ? 1 : 0];
     if (per_sm == 0 &&

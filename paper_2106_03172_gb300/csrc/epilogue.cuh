@@ -209,12 +209,12 @@ __device__ __forceinline__ void stage_views(const BackArgs &a, int vb, int nv, V
 }
 
 // Slice stacks: the pieces of a warp's list (offset, weight) times the values at base[i] +
-// offset, into sums of the even and the odd pieces: groups of 8 / W pieces, whose
-// loads are in flight together, then the rest as one group whose missing
-// pieces repeat the last one's load and are left out.
+// offset, in order: groups of 8 / W pieces, whose loads are in flight together,
+// then the rest as one group whose missing pieces repeat the last one's load
+// and are left out.
 template <int W>
 __device__ __forceinline__ void add_pieces(const float2 *piece, int np, const float *const (&base)[W],
-                                           float (&sum)[2][W]) {
+                                           float (&sum)[W]) {
     constexpr int U = 8 / W;
     int b = 0;
 #pragma unroll 1
@@ -230,7 +230,7 @@ __device__ __forceinline__ void add_pieces(const float2 *piece, int np, const fl
 #pragma unroll
         for (int u = 0; u < U; ++u)
 #pragma unroll
-            for (int i = 0; i < W; ++i) sum[u & 1][i] = fmaf(p[u].y, x[u][i], sum[u & 1][i]);
+            for (int i = 0; i < W; ++i) sum[i] = fmaf(p[u].y, x[u][i], sum[i]);
     }
     if (b < np) {
         float2 p[U];
@@ -245,7 +245,7 @@ __device__ __forceinline__ void add_pieces(const float2 *piece, int np, const fl
         for (int u = 0; u < U; ++u)
             if (b + u < np)
 #pragma unroll
-                for (int i = 0; i < W; ++i) sum[u & 1][i] = fmaf(p[u].y, x[u][i], sum[u & 1][i]);
+                for (int i = 0; i < W; ++i) sum[i] = fmaf(p[u].y, x[u][i], sum[i]);
     }
 }
 

@@ -28,9 +28,9 @@ namespace {
 // blocks fit on an SM (40 registers spill).
 constexpr int kFwdMinBlocks = 5;
 
-template <int CHUNKS, int MODE, bool LL, bool REF = false>
-__global__ void __launch_bounds__(kBlock, CHUNKS >= 32 ? kFwdMinBlocks : 5) forward_tile_kernel(const FwdArgs a) {
-    forward_tile_body<CHUNKS, MODE, LL, REF>(a, blockIdx.x);
+template <int CHUNKS, int MODE, bool LL>
+__global__ void __launch_bounds__(kBlock, kFwdMinBlocks) forward_tile_kernel(const FwdArgs a) {
+    forward_tile_body<CHUNKS, MODE, LL>(a, blockIdx.x);
 }
 
 // Persistent batched forward: a resident grid whose blocks claim work items
@@ -83,7 +83,6 @@ __global__ void __launch_bounds__(kBlock, kFwdMinBlocks)
                 if (sg.kind == WK_FWD_UPDATE) {
                     a.sub_off = m.sub_off;
                     a.t_dev = m.seq + iter;
-                    a.ref = m.ref;
                     a.img = in_is_img ? m.img : m.alt;
                     a.out = m.ratio;
                 } else if (sg.kind == WK_FWD_ANCHOR) {
@@ -151,9 +150,7 @@ __global__ void __launch_bounds__(kBlock) count_nnz_kernel(const FwdArgs a, unsi
 template <int CHUNKS>
 pet_status dispatch_tile(const FwdArgs &a, int mode, bool ll, int blocks, cudaStream_t s) {
     void (*k)(FwdArgs) = nullptr;
-    if (a.ref && mode == FWD_RATIO && !ll)
-        k = forward_tile_kernel<CHUNKS, FWD_RATIO, false, kRefRounding>;
-    else if (mode == FWD_YHAT && !ll)
+    if (mode == FWD_YHAT && !ll)
         k = forward_tile_kernel<CHUNKS, FWD_YHAT, false>;
     else if (mode == FWD_RATIO && !ll)
         k = forward_tile_kernel<CHUNKS, FWD_RATIO, false>;

@@ -269,34 +269,25 @@ int choose_group(const pet_plan *plan) {
     return plan->fwd_chunks > 0 ? plan->fwd_chunks : default_chunks(plan->nx, plan->ny);
 }
 
-// Band chunks per ray of a single-slice plan's subset and full-data forward
-// passes (anchor ratios, objectives, all-view projections).  A grid that fills
-// the GPU several times over is bound by instruction issue rather than latency,
-// and each thread's fixed work (ray set-up, chunk reduction, epilogue) is better
-// spread over more bands: the chunk count is halved, down to 16, while the grid
-// keeps at least kLargeGrid blocks.  Measured: 512^2 reconstruction with 60
-// views a subset 2180 us at 16 chunks against 2312 us at 32; a 256^2 subset of 9
-// views (207 blocks at 16 chunks) 157 us a SAGA epoch against 140 us at 32.  A
-// count the caller set or tuned is kept for the subsets.  Stacks and multi-ring
-// plans keep theirs.  Reference rounding (`ref`): the order of sums is part of
-// it, so subsets keep the plan's count and full passes at most kRefBands bands
-// a chunk.
+// Band chunks per ray of a full-data forward pass (anchor ratios, objectives,
+// all-view projections) of a single-slice plan.  Such a grid is large, so the
+// kernel is bound by instruction issue rather than latency, and each thread's
+// fixed work (ray set-up, chunk reduction, epilogue) is better spread over
+// more bands: the chunk count is halved from the plan's, down to 16, while the
+// grid keeps at least kLargeGrid blocks and a chunk keeps at most kFullBands
+// bands (8 chunks measured slower again on a 256^2 image: too few warps left
+// to hide the load latency; on 512^2 images, 32 bands per chunk made the full
+// pass 547 us against 426 us at the plan's 32 chunks, while 384^2 images, 24
+// bands per chunk at 16 chunks, took 155 us against 168 us at 32).  Stacks
+// and multi-ring plans keep theirs.
 constexpr int kLargeGrid = 8 * 152;
-constexpr int kRefBands = 24;
+constexpr int kFullBands = 24;
 
-int subset_group(const pet_plan *plan, bool ref) {
-    int g = choose_group(plan);
-    if (plan->nz != 1 || plan->ring || plan->fwd_chunks > 0 || ref) return g;
-    while (g > 16 && forward_blocks(plan->max_sub_views * plan->nb, 1, g / 2) >= kLargeGrid) g /= 2;
-    return g;
-}
-
-int full_group(const pet_plan *plan, bool ref) {
+int full_group(const pet_plan *plan) {
     int g = choose_group(plan);
     if (plan->nz != 1 || plan->ring) return g;
     const int major = std::max(plan->nx, plan->ny);
-    while (g > 16 && forward_blocks(plan->M, 1, g / 2) >= kLargeGrid &&
-           (!ref || (major + g / 2 - 1) / (g / 2) <= kRefBands))
+    while (g > 16 && forward_blocks(plan->M, 1, g / 2) >= kLargeGrid && (major + g / 2 - 1) / (g / 2) <= kFullBands)
         g /= 2;
     return g;
 }

@@ -67,13 +67,11 @@ extern "C" pet_status pet_objective_noalloc(const pet_plan *plan, const float *d
     // ray's expected count is the one pet_objective computes
     const int group = full_group(plan);
     const int n_ll = forward_blocks(plan->M, plan->nz, group);
-    // the sizes refused are those of the finer chunks (the reference rounding's rule)
-    const int n_max = forward_blocks(plan->M, plan->nz, full_group(plan, true));
     const long long plane = (long long)plan->N * plan->nz;
     const long long n_pen = (plane + 255) / 256;
-    if ((long long)n_max + n_pen > kNoallocPartials)
+    if ((long long)n_ll + n_pen > kNoallocPartials)
         return set_error(PET_ERR_INVALID, "pet_objective_noalloc: image/sinogram too large for its fixed scratch (" +
-                                              std::to_string((long long)n_max + n_pen) + " block partials needed, " +
+                                              std::to_string((long long)n_ll + n_pen) + " block partials needed, " +
                                               std::to_string(kNoallocPartials) + " available)");
     double *scratch = nullptr;
     const pet_status st = scratch_for_plan_device(plan, &scratch);

@@ -9,7 +9,6 @@
 #include <cmath>
 #include <cstdint>
 #include <cstdlib>
-#include <mutex>
 #include <string>
 #include <utility>
 #include <vector>
@@ -55,13 +54,8 @@ struct alignas(16) ViewParams {
     float inv_du; // 1 / du (0 if du == 0), for band ranges only
     float uc0;    // centred minor coordinate of bin 0 at the central major line (approx.)
     int col;      // 1: major axis is x (columns); 0: major axis is y (rows)
-    float inv_adu; // 1 / |du| (kAxisInv if du == 0), for the piece shares
-    float pad[2];
+    float pad[3];
 };
-
-// inv_adu of an axis-aligned view: a share saturates to 0 or 1 for any offset
-// from a pixel edge above 1 / kAxisInv, and products with it stay finite.
-constexpr float kAxisInv = 1e30f;
 
 // Adding kRound to a float of magnitude below 2^22 leaves its integer part in
 // the low mantissa bits, rounded the way the addition rounds: the integer as
@@ -116,25 +110,17 @@ __device__ __forceinline__ void band_split(const ViewParams &vp, float va, float
     }
 }
 
-// band_split() with the floor by a directed-rounding add: the same weights,
-// bit for bit (the results of comparisons and roundings do not change), and
-// kRound + floor(lo) in place of the floor.
-__device__ __forceinline__ float band_split_ref(const ViewParams &vp, float va, float vb, float &w0, float &w1) {
-    const float lo = fminf(va, vb);
+// band_split() with the floor by a directed-rounding add, given the band's ends
+// in order: the same weights, bit for bit.  Returns kRound + floor(lo).  (An
+// ulp in a weight re-draws the rounding of every later iterate, so the
+// projectors of all kernels and launch shapes keep these expressions.)
+__device__ __forceinline__ float band_weights(float L, float Lm, float lo, float hi, float &w0, float &w1) {
     const float t = __fadd_rd(lo, kRound);
     const float fl1 = t - (kRound - 1.0f);
-    const float part = fminf((fl1 - lo) * vp.Lm, vp.L);
-    w0 = fmaxf(va, vb) <= fl1 ? vp.L : part;
-    w1 = vp.L - w0;
+    const float part = fminf((fl1 - lo) * Lm, L);
+    w0 = hi <= fl1 ? L : part;
+    w1 = L - w0;
     return t;
-}
-
-// Share of a band (as a fraction of its length) in the lower of the two minor
-// pixels it can touch, for the band's lower end `lo` and fl1 = floor(lo) + 1:
-// the line covers inv_adu of a band per pixel of minor displacement, so the
-// lower pixel gets min((fl1 - lo) / |du|, 1) and the upper one the rest.
-__device__ __forceinline__ float band_share(float fl1, float lo, float inv_adu) {
-    return __saturatef((fl1 - lo) * inv_adu);
 }
 
 // ---------------------------------------------------------------------------
@@ -260,15 +246,6 @@ cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, s
 // ---------------------------------------------------------------------------
 // Kernel argument blocks.
 // ---------------------------------------------------------------------------
-// Which rounding a single-slice projection takes.  A BF16 table keeps 8 bits
-// of each subset gradient, so an ulp in a projection moves the entries that lie
-// on a rounding boundary by 2^-8 of themselves (measured: 2.5e-5 of an image
-// after three updates, where FP32 states stay within 1e-6).  States with such
-// a table, and the sensitivities their entries subtract, therefore keep the
-// rounding of band_split() and the order of its sums bit for bit; all others
-// take the cheaper band_share() form, which is as close to the exact weights.
-constexpr bool kRefRounding = true;
-
 enum FwdMode { FWD_NONE = 0, FWD_YHAT = 1, FWD_RATIO = 2 };
 
 struct FwdArgs {
@@ -291,7 +268,6 @@ struct FwdArgs {
     float *out;               // compact output (yhat or ratio)
     double *ll_partials;      // per-block partial log-likelihood (LL only)
     int *status;              // device error latch (may be null)
-    int ref;                  // single slices: kRefRounding
 };
 
 // View range of a forward launch: given on the host, or (t_dev set) read on
@@ -364,12 +340,10 @@ struct BackArgs {
     const int *sub_off;   // view offsets of subsets in `order`
     int t0;               // subset of blockIdx.y == 0
     const int *t_dev;     // if set: the subset index is read here (grid.y must be 1)
-    int bw;               // single-slice tile kernel: bins staged per view of a tile (tile_bins)
-    int cand1, cand2;     // and the most candidate bins of a pixel, of a pair of pixels
     int cands, cand_rounds;   // slice stacks: lanes per view, 32-bin pieces per view
-    int ref;              // single slices, EPI_ANCHOR: kRefRounding
     int r_view0;          // view position of r[0] (ignored when t_dev is set: r is
                           //   then the compact ratio of subset *t_dev)
+    int bw, cand;         // single-slice tile kernel: bins staged per view, most candidates of a pixel
     int nx, ny, nz, nb, ns;  // nz: image entries per pixel (slices, or layers when axial)
     int axial;            // multi-ring: layers are coupled (6-neighbourhood penalty) and the
                           //   sensitivities are per voxel ([ns][nx*ny*nz]); else per pixel
@@ -407,7 +381,7 @@ struct BatchMember {
     int nx, ny, nb, ns;
     unsigned nb_mul;       // division by nb (FwdArgs)
     int nb_shift;
-    int bw, cand1, cand2;  // back-projection tiles (BackArgs)
+    int bw, cand;          // back-projection tiles (BackArgs)
     const float *sens_t;
     const float *sens;
     const float *g;
@@ -418,7 +392,6 @@ struct BatchMember {
     float delta;
     int *status;
     int algo, table_dtype;
-    int ref;               // kRefRounding
     float *img, *alt, *ratio;
     float *ratio_full;     // anchor-pass ratio over all views (SVREM, SVRG), subset-major
     float *s_hat;
@@ -523,7 +496,7 @@ struct pet_plan {
     int device;
     int fwd_chunks = 0;             // single-slice forward: band chunks per ray (8, 16 or 32)
     int back_run = 8;               // the caller's choice (4 or 8); no launch shape depends on it
-    int bw = 0, cand1 = 0, cand2 = 0;   // single-slice back projection (BackArgs)
+    int bw = 0, cand = 0;           // single-slice back projection (BackArgs)
     int cands = 1, cand_rounds = 1;     // slice stacks (BackArgs)
     unsigned nb_mul = 0;            // division of a ray index by nb (bins_division)
     int nb_shift = 0;
@@ -538,9 +511,6 @@ struct pet_plan {
     int *d_all_off = nullptr;       // {0, na}
     float *d_sens_t = nullptr;      // [ns][N]
     float *d_sens = nullptr;        // [N]
-    mutable float *d_sens_t_ref = nullptr;   // [ns + 1][N]: d_sens_t and d_sens in the reference
-                                             //   rounding, once a state needs them
-    mutable std::mutex ref_mu;      // guards d_sens_t_ref
     float4 *d_lz = nullptr;         // multi-ring: axial table per line [view][bin][pair]
 };
 
@@ -564,7 +534,6 @@ struct pet_batch;
 struct pet_state {
     const pet_problem *prob;
     int algo, table_dtype;
-    int ref;               // kRefRounding
     float *img;                     // caller's image (current iterate)
     float *alt = nullptr;           // ping-pong partner
     float *ratio = nullptr;         // [max subset rays * nz]
@@ -602,7 +571,6 @@ struct pet_batch {
         int kind;                   // 0 forward, 1 back + update (GENPOT 0/1 in `genpot`), 2 anchor finishes
         int seg_off, n_segs, n_items;
         int genpot;                 // back: general-potential epilogues
-        int ref;                    // back: members with the reference rounding
         int claim;                  // claim counter slot
     };
     std::vector<std::vector<Phase>> phases;   // [n_iter]
@@ -663,8 +631,7 @@ pet_status launch_forward(const FwdArgs &a, int mode, bool ll, int group, cudaSt
                           int *n_blocks_out, int rays_for_grid = -1);
 int forward_blocks(int n_rays, int nz, int group);
 int choose_group(const pet_plan *plan);
-int subset_group(const pet_plan *plan, bool ref = false);   // band chunks of subset passes
-int full_group(const pet_plan *plan, bool ref = false);     // and of full-data passes
+int full_group(const pet_plan *plan);     // band chunks of a full-data single-slice pass
 int default_chunks(int nx, int ny);
 pet_status launch_back(const BackArgs &a, int epi, int table_dtype, int n_subsets_grid,
                        cudaStream_t s, int max_views);
@@ -684,9 +651,9 @@ pet_status launch_count_nnz(const FwdArgs &a, unsigned long long *d_count, cudaS
 // ratio kinds (WK_FWD_UPDATE, WK_FWD_ANCHOR), true the log-likelihood kind.
 pet_status launch_persistent_forward(const BatchMember *d_members, const WorkSeg *d_segs, int n_segs, int n_items,
                                      int iter, int in_is_img, int *claim, bool objective, cudaStream_t s);
-void tile_bins(double pixel_mm, double bin_mm, int nb, int nx, int ny, int &bw, int &cand1, int &cand2);   // BackArgs
+void tile_bins(double pixel_mm, double bin_mm, int nb, int nx, int ny, int &bw, int &cand);   // BackArgs
 pet_status launch_persistent_back(const BatchMember *d_members, const WorkSeg *d_segs, int n_segs, int n_items,
-                                  int iter, int in_is_img, int *claim, bool general_potential, bool ref, cudaStream_t s);
+                                  int iter, int in_is_img, int *claim, bool general_potential, cudaStream_t s);
 pet_status launch_zero_ints(int *p, int n, cudaStream_t s);
 // Dependency-driven batched epoch (dataflow.cu): the whole list in one launch.
 pet_status launch_dataflow_epoch(const BatchMember *d_members, const DfSeg *d_segs, int n_segs, int n_items,

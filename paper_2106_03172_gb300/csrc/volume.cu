@@ -151,17 +151,15 @@ __global__ void __launch_bounds__(kBlock) forward_slim_kernel(const FwdArgs a) {
 // Slice-stack forward: the geometry is shared by every slice.  A warp takes one
 // ray and a window of 32 W consecutive slices, lane l the slices l, l + 32, ...
 // of the window, so a load instruction reads 32 consecutive floats of one
-// pixel's slice column ([iy][ix][z] layout).  For kStackBands bands of the ray at
-// a time, lane l evaluates the bands l, l + 32, ... once for all slices, and the
-// nonzero pieces go to a list in shared memory, in band order, which the warp
-// then walks (the same pieces for every lane) into two sums, even and odd
-// pieces (deterministic).
+// pixel's slice column ([iy][ix][z] layout).  The ray's bands form kStackChunks
+// chunks; for up to kStackBands bands of a chunk at a time, lane l evaluates the
+// bands l, l + 32, ... once for all slices, and the nonzero pieces go to a list
+// in shared memory, in band order, which the warp then walks (the same pieces
+// for every lane).  Pieces are added in order within a chunk and the chunk sums
+// pairwise, so the result is deterministic.
 //
 // Bound by instruction issue (seven instructions per piece and two windows of
-// slices) and the gathers' L1 wavefronts.  47 slices of 128^2, 252 views of 344
-// bins (ncu), against 8 z-lanes x 4 chunks (forward_slim_kernel's layout): full
-// ratio pass 263 -> 170 us (183M -> 118M warp instructions, L1 wavefronts 85% ->
-// 66%), a subset 29.4 -> 22.1 us.
+// slices) and the gathers' L1 wavefronts.
 constexpr int kStackBands = 128;
 
 template <int MODE, bool LL, int W>
@@ -198,8 +196,12 @@ __global__ void __launch_bounds__(kBlock, 4) forward_stack_kernel(const FwdArgs 
         const float *img[W];
 #pragma unroll
         for (int i = 0; i < W; ++i) img[i] = a.img + min(z0 + 32 * i, a.nz - 1);
-        for (int kseg = k_lo; kseg < k_hi; kseg += kStackBands) {
-            const int ke = min(k_hi, kseg + kStackBands);
+        const int per = (n_major + kStackChunks - 1) / kStackChunks;
+        float part[W] = {};                                // the chunk's sum so far
+        for (int kseg = k_lo; kseg < k_hi;) {
+            // bands to the end of the chunk, at most kStackBands
+            const int c = kseg / per;
+            const int ke = min(min(k_hi, (c + 1) * per), kseg + kStackBands);
             int np = 0;
             __syncwarp();
             for (int kbase = kseg; kbase < ke; kbase += 32) {
@@ -208,7 +210,8 @@ __global__ void __launch_bounds__(kBlock, 4) forward_stack_kernel(const FwdArgs 
                 int o = 0;
                 if (k < ke) {
                     const float kc = (float)k - hm;
-                    const float t = band_split_ref(vp, band_point(vp, u.y, kc), band_point(vp, u.y, kc + 1.0f), w0, w1);
+                    const float va = band_point(vp, u.y, kc), vb = band_point(vp, u.y, kc + 1.0f);
+                    const float t = band_weights(vp.L, vp.Lm, fminf(va, vb), fmaxf(va, vb), w0, w1);
                     const int m0 = (int)(__float_as_uint(t) - kRoundBits) + ui;
                     o = k * s_major + m0 * s_minor;
                     if ((unsigned)m0 >= (unsigned)n_minor) w0 = 0.0f;
@@ -222,7 +225,14 @@ __global__ void __launch_bounds__(kBlock, 4) forward_stack_kernel(const FwdArgs 
                 np += __popc(has0) + __popc(has1);
             }
             __syncwarp();
-            add_pieces<W>(piece, np, img, sum);
+            add_pieces<W>(piece, np, img, part);
+            if (ke == k_hi || ke == (c + 1) * per)
+#pragma unroll
+                for (int i = 0; i < W; ++i) {
+                    if (c < kStackChunks / 2) sum[0][i] += part[i]; else sum[1][i] += part[i];
+                    part[i] = 0.0f;
+                }
+            kseg = ke;
         }
     }
 

@@ -104,9 +104,8 @@ __global__ void __launch_bounds__(kBlock) back_slim_kernel(const BackArgs a) {
 // bin's slice column ([view][bin][z]).  The lanes share the candidate bins of
 // the subset's views among them (a.cands per view), evaluate each one's band
 // piece once for all slices, and leave the nonzero weights, in view and bin
-// order, in shared memory; the warp then walks that list into two sums, even and
-// odd pieces (deterministic), and each lane applies the update to its own
-// slices.  Bound by instruction issue.  47 slices of 128^2 (ncu), against 4
+// order, in shared memory; the warp then walks that list in order
+// (deterministic), and each lane applies the update to its own slices.  Bound by instruction issue.  47 slices of 128^2 (ncu), against 4
 // pixels x 8 z-lanes (back_slim_kernel's layout): anchor of 14 subsets 290 -> 231
 // us, an update 37.5 -> 32.1 us; 24 slices of 96^2, a run call 723 -> 440 us.
 constexpr int kStackPieces = 96;     // list entries per warp (a round adds up to 32)
@@ -136,7 +135,7 @@ __global__ void __launch_bounds__(kBlock, 5) back_stack_kernel(const BackArgs a)
     const int iy = n / a.nx;
     const int z0 = win * 32 * W + lane;                   // this lane's first slice
 
-    float acc[2][W] = {};
+    float acc[W] = {};
     // a lane past the last slice reads that slice again and drops the sum
     const float *r[W];
 #pragma unroll
@@ -165,7 +164,8 @@ __global__ void __launch_bounds__(kBlock, 5) back_stack_kernel(const BackArgs a)
             if (j <= jhi) {
                 const float2 u = __ldg(a.uc + s_vid[q] * a.nb + j);
                 float w0, w1;
-                const float t = band_split_ref(vp, band_point(vp, u.y, kc), band_point(vp, u.y, kc + 1.0f), w0, w1);
+                const float e0 = band_point(vp, u.y, kc), e1 = band_point(vp, u.y, kc + 1.0f);
+                const float t = band_weights(vp.L, vp.Lm, fminf(e0, e1), fmaxf(e0, e1), w0, w1);
                 const int c0 = (int)(__float_as_uint(t) - kRoundBits) + (int)u.x;
                 w = (c0 == mrel) ? w0 : ((c0 + 1 == mrel) ? w1 : 0.0f);
                 off = ((vb + q - r_view0) * a.nb + j) * a.nz;
@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(kBlock, 5) back_stack_kernel(const BackArgs a)
     for (int i = 0; i < W; ++i) {
         const int z = z0 + 32 * i;
         if (z < a.nz)
-            apply_epilogue<EPI, TQ, GENPOT>(a, t, (long long)n * a.nz + z, n, ix, iy, z, acc[0][i] + acc[1][i]);
+            apply_epilogue<EPI, TQ, GENPOT>(a, t, (long long)n * a.nz + z, n, ix, iy, z, acc[i]);
     }
 }
 
