@@ -12,7 +12,7 @@ namespace petvr {
 namespace {
 
 constexpr int kBlock = 256;
-constexpr int kLanes = 4;           // multi-ring volumes: lanes per pixel column or voxel
+constexpr int kLanes = 4;           // tall multi-ring volumes: lanes per voxel
 constexpr float kCandEps = 1e-3f;   // candidate-bin margin (pixels)
 
 // A float that may have been written earlier in the same kernel launch by

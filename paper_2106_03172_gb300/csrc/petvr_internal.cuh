@@ -161,6 +161,26 @@ __device__ __forceinline__ float layer_fraction(float za, float zb, int iz) {
     return ov > 0.0f ? __fdividef(ov, hi - lo) : 0.0f;
 }
 
+// Calls add(layer, share) for every layer of [0, L) that the axial range between
+// za and zb crosses, with its share of the range (layer_fraction).  Nearly every
+// range lies within one layer: that case takes no loop (the share is
+// layer_fraction's own quotient, so the bits are the same).
+template <class Add>
+__device__ __forceinline__ void piece_layers(float za, float zb, int L, Add &&add) {
+    const float lo = fminf(za, zb), hi = fmaxf(za, zb);
+    const float t = __fadd_rd(lo, kRound);
+    // kRound's integers hold below 2^22; other ranges take the general loop
+    if (t == __fadd_rd(hi, kRound) && lo >= 0.0f && hi < fminf((float)L, 4194304.0f)) {
+        add((int)(__float_as_uint(t) - kRoundBits), hi > lo ? __fdividef(hi - lo, hi - lo) : 1.0f);
+        return;
+    }
+    const int il = max(0, (int)floorf(lo)), ih = min(L - 1, (int)floorf(hi));
+    for (int iz = il; iz <= ih; ++iz) {
+        const float fr = layer_fraction(za, zb, iz);
+        if (fr > 0.0f) add(iz, fr);
+    }
+}
+
 // Nonnegative root of a/f - 2 b f + c = 0 (the surrogate M-step of §3,
 // Eq. (svrsurder)); cancellation-free in both signs of c, b = 0 allowed;
 // 0 when S <= 0 or a <= 0 (zero-denominator remedy of §2.3).

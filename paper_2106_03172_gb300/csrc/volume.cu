@@ -308,9 +308,9 @@ __global__ void __launch_bounds__(kBlock) ring_forward_kernel(const FwdArgs a) {
         float va = band_point(vp, u.y, kc);
         for (int k = kb; k < ke; ++k) {
             const float vb = band_point(vp, u.y, kc + 1.0f);
-            float fl, w0, w1;
-            band_split(vp, va, vb, fl, w0, w1);
-            const int m0 = (int)fl + ui;
+            float w0, w1;
+            const float t = band_weights(vp.L, vp.Lm, fminf(va, vb), fmaxf(va, vb), w0, w1);
+            const int m0 = (int)(__float_as_uint(t) - kRoundBits) + ui;
 #pragma unroll
             for (int side = 0; side < 2; ++side) {
                 const int m = m0 + side;
@@ -322,14 +322,10 @@ __global__ void __launch_bounds__(kBlock) ring_forward_kernel(const FwdArgs a) {
 #pragma unroll
                 for (int pr = 0; pr < P; ++pr) {
                     const float4 lz = __ldg(lzr + pr);
-                    const float za = piece_zeta(lz, kc, f_lo), zb = piece_zeta(lz, kc, f_hi);
                     const float wl = w * lz.z;
-                    const int il = max(0, (int)floorf(fminf(za, zb)));
-                    const int ih = min(L - 1, (int)floorf(fmaxf(za, zb)));
-                    for (int iz = il; iz <= ih; ++iz) {
-                        const float fr = layer_fraction(za, zb, iz);
-                        if (fr > 0.0f) acc[pr] = fmaf(wl * fr, __ldg(colp + iz), acc[pr]);
-                    }
+                    piece_layers(piece_zeta(lz, kc, f_lo), piece_zeta(lz, kc, f_hi), L, [&](int iz, float fr) {
+                        acc[pr] = fmaf(wl * fr, __ldg(colp + iz), acc[pr]);
+                    });
                 }
             }
             va = vb;
