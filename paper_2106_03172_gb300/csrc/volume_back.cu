@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(kBlock) ring_back_kernel(const BackArgs a) {
 // Bound by instruction issue and, on subset launches, by the launch's latency.
 // Against four lanes per column on a view each (diverging) and a loop over the
 // layers with a division each: an SVREM epoch of the 2-ring 128^2 x 3 volume
-// 879 -> 687 us, of 4 layers and 2 rings at 64^2 (random problem) 363 -> 221 us.
+// 879 -> 687 us.
 constexpr int kColumns = 64;
 constexpr int kViewLanes = kBlock / kColumns;
 
