@@ -33,20 +33,17 @@ namespace petvr {
 
 namespace {
 
-// Launches over this many views at once and no state's update (all-view back
-// projections) split them over kViewGroups groups of threads per tile.
-constexpr int kManyViews = 32;
 constexpr int kBackMinBlocks = 4;
 
-template <int EPI, typename TQ, bool GENPOT, int GROUPS = 1>
-__global__ void __launch_bounds__(kBlock *GROUPS, kBackMinBlocks / GROUPS) back_tile_kernel(const BackArgs a) {
+template <int EPI, typename TQ, bool GENPOT>
+__global__ void __launch_bounds__(kBlock, kBackMinBlocks) back_tile_kernel(const BackArgs a) {
     const int t = a.t_dev ? __ldg(a.t_dev) : a.t0 + (int)blockIdx.y;
-    back_tile_body<EPI, TQ, GENPOT, false, GROUPS>(a, t, blockIdx.x);
+    back_tile_body<EPI, TQ, GENPOT>(a, t, blockIdx.x);
 }
 
-template <int EPI, typename TQ, bool GENPOT>
-__global__ void __launch_bounds__(kBlock) back_run_kernel(const BackArgs a) {
-    back_run_body<EPI, TQ, GENPOT>(a, a.t0 + (int)blockIdx.y, blockIdx.x);
+template <int EPI, typename TQ, bool GENPOT, int NT = kBlock>
+__global__ void __launch_bounds__(NT) back_run_kernel(const BackArgs a) {
+    back_run_body<EPI, TQ, GENPOT, NT>(a, a.t0 + (int)blockIdx.y, blockIdx.x);
 }
 
 // Persistent batched back projection + update: a resident grid whose blocks
@@ -145,9 +142,9 @@ __global__ void __launch_bounds__(kBlock, kBackMinBlocks)
 // blocks are placed while the kernel ahead still runs, and pile up on the SMs
 // that have room, up to the register limit of four, while others stay empty:
 // the fullest SM sets the time.  Bounded to one above the even share; a tighter
-// bound (256^2: 131 us a SAGA epoch instead of 140) costs launches of several
-// streams more (the four-method step 1969 us instead of 1800), none 153 and
-// 1750 us; at an even share of three and more the register limit does.
+// bound was faster alone and slower with several streams.  256^2: a SAGA epoch
+// 160 us (no bound: 176), the four-method step on four streams 2055 us (1994);
+// at an even share of three and more the register limit does.
 size_t residency_smem(const void *kernel, int blocks, size_t base) {
     const int cap = (blocks + sm_count() - 1) / sm_count() + 1;
     if (cap > 3) return base;
@@ -168,20 +165,31 @@ struct TileBack {
     cudaStream_t s;
     int max_views;
 
+    template <int EPI, typename TQ, bool GENPOT, int NT>
+    pet_status run_launch(dim3 grid) const {
+        launch_dependent(back_run_kernel<EPI, TQ, GENPOT, NT>, grid, dim3(NT), run_smem_bytes<NT>(), s, a);
+        return check_launch("back_run_kernel");
+    }
+
     template <int EPI, typename TQ, bool GENPOT>
     pet_status run() const {
         const int tiles = ((a.nx + kTile - 1) / kTile) * ((a.ny + kTile - 1) / kTile);
         const dim3 grid((unsigned)tiles, (unsigned)ny_grid);
-        if constexpr (EPI == EPI_ANCHOR || EPI == EPI_SAGA_INIT || EPI == EPI_SAGAEM_INIT) {
-            launch_dependent(back_run_kernel<EPI, TQ, GENPOT>, grid, dim3(kBlock), run_smem_bytes(), s, a);
-            return check_launch("back_run_kernel");
+        if constexpr (EPI == EPI_ANCHOR || EPI == EPI_SAGA_INIT || EPI == EPI_SAGAEM_INIT)
+            return run_launch<EPI, TQ, GENPOT, kBlock>(grid);
+        // Plain back projections (no update behind them): runs, one per thread and
+        // pass.  Forward + back, 512 threads against staged bins (bins = pixels):
+        // 300^2 x 270 views 131.9 us (140.5), 300^2 x 30 18.6 (18.2), 477x461 x 30
+        // 33.5 (30.1), 512^2 x 500 648 (581); bins of 2/3 of a pixel 182 (225),
+        // 24.6 (29.2), 45.7 (47.0), 885 (896).  Where at most two blocks share an
+        // SM and there are several passes, 1024 threads: 213x199 x 220 views
+        // 72.7 us (512 threads 89.8, staged bins 92.5); with 300^2 x 270's 361
+        // tiles 139.9 (512: 131.9), with 28 views 15.8 (15.6).
+        if constexpr (EPI == EPI_PLAIN) {
+            if (tiles * ny_grid <= 2 * sm_count() && max_views > 2 * kRunViews<1024>)
+                return run_launch<EPI, TQ, GENPOT, 1024>(grid);
+            return run_launch<EPI, TQ, GENPOT, 512>(grid);
         }
-        if constexpr (EPI == EPI_PLAIN)
-            if (max_views >= kManyViews) {
-                launch_dependent(back_tile_kernel<EPI, TQ, GENPOT, kViewGroups>, grid, dim3(kBlock * kViewGroups),
-                                 tile_smem_bytes(), s, a);
-                return check_launch("back_tile_kernel");
-            }
         const auto k = back_tile_kernel<EPI, TQ, GENPOT>;
         const size_t smem = tile_smem_bytes();
         launch_dependent(k, grid, dim3(kBlock), a.t_dev ? residency_smem((const void *)k, tiles, smem) : smem, s, a);

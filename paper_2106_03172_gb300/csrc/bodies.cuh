@@ -205,7 +205,6 @@ __device__ __forceinline__ void forward_item(const FwdArgs &a, int shape, int bx
 // then over the views, so the result is deterministic and needs no atomics.
 constexpr int kStageViews = 32;        // views per pass
 constexpr int kStageBins = 1024;       // staged bins per pass
-constexpr int kViewGroups = 4;         // groups of threads on launches over all views
 constexpr int kUnrolledCand = 3;       // largest candidate count with a loop of its own
 
 // Per-view constants of a tile.  A ray's offset from pixel m at its band's
@@ -284,18 +283,13 @@ __device__ __forceinline__ void stage_bins(int nq, int bw, Load &&load) {
 // arrive in one, and the views' chains overlap.  The weights are band_weights()
 // of the positions the forward computes, bit for bit (the ends come in order,
 // so the floor, the share and the test of the upper end are all there is to a
-// candidate).  Against runs of 8 pixels a thread (back_run_body): two 256^2 SVREM
-// epochs 601 -> 534 us, a 512^2 reconstruction 3400 -> 3131 us.
-//
-// GROUPS > 1: group g of the block's threads takes the views g, g + GROUPS, ...
-// of a pass, and the groups' sums are added in order (launches over all views,
-// whose few tiles would otherwise walk every view one after another).
-template <int EPI, typename TQ, bool GENPOT, bool COH = false, int GROUPS = 1>
+// candidate).  Against runs of 8 pixels a thread (back_run_body), same bound on the
+// blocks per SM: a 201x147 SVRG run 418 -> 373 us, a 512^2 reconstruction 3400 ->
+// 3131, a 256^2 SAGA epoch 163 -> 160, two SVREM epochs 522 -> 534.
+template <int EPI, typename TQ, bool GENPOT, bool COH = false>
 __device__ __forceinline__ void back_tile_body(const BackArgs &a, const int t, const int bx) {
     constexpr int NT = kTile * kTile;
     extern __shared__ unsigned char smem_raw[];
-    const int tid = GROUPS > 1 ? threadIdx.x % NT : threadIdx.x;
-    const int group = GROUPS > 1 ? threadIdx.x / NT : 0;
     TileShared &sh = *reinterpret_cast<TileShared *>(smem_raw);
     const int vb = __ldg(a.sub_off + t);
     const int nv = __ldg(a.sub_off + t + 1) - vb;
@@ -303,7 +297,7 @@ __device__ __forceinline__ void back_tile_body(const BackArgs &a, const int t, c
     const int tiles_x = (a.nx + kTile - 1) / kTile;
     const int x0 = (bx % tiles_x) * kTile;
     const int y0 = (bx / tiles_x) * kTile;
-    const int tx = tid % kTile, ty = tid / kTile;
+    const int tx = threadIdx.x % kTile, ty = threadIdx.x / kTile;
     const bool staged = a.bw <= kStageBins;      // else (bins far finer than pixels) bins are read in place
     const int per_pass = staged ? min(kStageViews, kStageBins / a.bw) : kStageViews;
     const float mx = (float)(x0 + tx - (a.nx >> 1)), my = (float)(y0 + ty - (a.ny >> 1));
@@ -318,13 +312,13 @@ __device__ __forceinline__ void back_tile_body(const BackArgs &a, const int t, c
         }
         __syncthreads();
         // plan constants before the wait for the kernel ahead, ratios after it
-        for (int i = threadIdx.x; i < nq * kTile; i += NT * GROUPS) {
+        for (int i = threadIdx.x; i < nq * kTile; i += NT) {
             const TileView &tv = sh.views[i / kTile];
             const float kc = tv.k0 + (float)(i % kTile);
             sh.bands[i] = make_float4(kc, fmaf(-(kc * tv.du), tv.invK, tv.cst), tv.invK, kc + tv.step);
         }
         if (staged)
-            stage_bins<NT * GROUPS>(nq, a.bw, [&](int q, int i, int e, bool live) {
+            stage_bins<NT>(nq, a.bw, [&](int q, int i, int e, bool live) {
                 const int j = sh.views[q].j0 + i;
                 float2 u = make_float2(0.0f, 0.0f);
                 if (live && (unsigned)j < (unsigned)a.nb) u = __ldg(a.uc + sh.views[q].v * a.nb + j);
@@ -337,7 +331,7 @@ __device__ __forceinline__ void back_tile_body(const BackArgs &a, const int t, c
             pdl_trigger();
         }
         if (staged)
-            stage_bins<NT * GROUPS>(nq, a.bw, [&](int q, int i, int e, bool live) {
+            stage_bins<NT>(nq, a.bw, [&](int q, int i, int e, bool live) {
                 const int j = sh.views[q].j0 + i;
                 float r = 0.0f;
                 if (live && (unsigned)j < (unsigned)a.nb)
@@ -353,7 +347,7 @@ __device__ __forceinline__ void back_tile_body(const BackArgs &a, const int t, c
         auto gather = [&](auto nc) {
             constexpr int NC = decltype(nc)::value;
 #pragma unroll (NC == 2 ? 2 : 1)
-            for (int q = group; q < nq; q += GROUPS) {
+            for (int q = 0; q < nq; ++q) {
                 const float2 vc = *reinterpret_cast<const float2 *>(&sh.views[q].du);       // du, du_lo
                 const float4 vd = *reinterpret_cast<const float4 *>(&sh.views[q].L);        // L, Lm, base, flags
                 const int flags = __float_as_int(vd.w);
@@ -403,15 +397,6 @@ __device__ __forceinline__ void back_tile_body(const BackArgs &a, const int t, c
             gather(std::integral_constant<int, 0>());
     }
     pdl_wait();   // returns at once after the wait above; covers an empty subset
-    if constexpr (GROUPS > 1) {
-        float *sums = reinterpret_cast<float *>(smem_raw);      // [GROUPS][NT]
-        __syncthreads();
-        if (group > 0) sums[group * NT + tid] = acc;
-        __syncthreads();
-        if (group > 0) return;
-#pragma unroll
-        for (int g = 1; g < GROUPS; ++g) acc += sums[g * NT + tid];
-    }
     const int ix = x0 + tx, iy = y0 + ty;
     if (ix < a.nx && iy < a.ny) {
         const int n = iy * a.nx + ix;
@@ -419,32 +404,39 @@ __device__ __forceinline__ void back_tile_body(const BackArgs &a, const int t, c
     }
 }
 
-// All-subset launches (anchors, table fills), which fill the GPU: for each view,
-// the tile's bands are cut into runs of kRun pixels along the view's minor
+// All-subset launches (anchors, table fills) and plain back projections: for each
+// view, the tile's bands are cut into runs of kRun pixels along the view's minor
 // axis; one thread walks the rays that can cross a run in order and adds each
 // ray's two band pieces into per-view partial sums in shared memory (every
 // (view, pixel) slot has exactly one writer, so no atomics).  Then each thread
 // sums its pixel's partials over the views in order.  The same weights and
 // order of sums as back_tile_body, bit for bit, in fewer instructions (a band
 // is evaluated once for the run, not for every pixel it can touch) but a longer
-// chain: 256^2, 21 subsets ANCHOR_TIMES.
+// chain: 256^2, 21 subsets 40 us and 29.7M warp instructions, staged bins 43 us
+// and 35.3M (ncu).
 constexpr int kRun = 8;
-constexpr int kRunViews = 16;          // views per shared-memory pass
 
+// Views per shared-memory pass of an NT-thread block: a run per thread at 512
+// threads and more, two per thread at 256.
+template <int NT>
+constexpr int kRunViews = NT > 512 ? NT / 32 : 16;
+
+template <int VIEWS>
 struct RunShared {
-    float part[kRunViews][kTile * kTile];
-    ViewParams views[kRunViews];
-    int vid[kRunViews];
+    float part[VIEWS][kTile * kTile];
+    ViewParams views[VIEWS];
+    int vid[VIEWS];
 };
 
-template <int EPI, typename TQ, bool GENPOT>
+template <int EPI, typename TQ, bool GENPOT, int NT>
 __device__ __forceinline__ void back_run_body(const BackArgs &a, const int t, const int bx) {
     extern __shared__ unsigned char smem_raw[];
-    RunShared &sh = *reinterpret_cast<RunShared *>(smem_raw);
+    constexpr int kViews = kRunViews<NT>;
+    RunShared<kViews> &sh = *reinterpret_cast<RunShared<kViews> *>(smem_raw);
     const int vb = __ldg(a.sub_off + t);
     const int nv = __ldg(a.sub_off + t + 1) - vb;
     const int r_view0 = a.t_dev ? vb : a.r_view0;
-    constexpr int nthr = kBlock;
+    constexpr int nthr = NT;                      // >= kTile * kTile
 
     const int tiles_x = (a.nx + kTile - 1) / kTile;
     const int x0 = (bx % tiles_x) * kTile;
@@ -453,8 +445,8 @@ __device__ __forceinline__ void back_run_body(const BackArgs &a, const int t, co
     constexpr int kRunsPerView = kTile * kRunsPerBand;
 
     float acc = 0.0f;
-    for (int q0 = 0; q0 < nv; q0 += kRunViews) {
-        const int nq = min(kRunViews, nv - q0);
+    for (int q0 = 0; q0 < nv; q0 += kViews) {
+        const int nq = min(kViews, nv - q0);
         for (int q = threadIdx.x; q < nq; q += nthr) {
             const int v = __ldg(a.order + vb + q0 + q);
             sh.vid[q] = v;
@@ -504,19 +496,23 @@ __device__ __forceinline__ void back_run_body(const BackArgs &a, const int t, co
             }
         }
         __syncthreads();
-        for (int ql = 0; ql < nq; ++ql) acc += sh.part[ql][threadIdx.x];
+        if (NT == kTile * kTile || threadIdx.x < kTile * kTile)
+            for (int ql = 0; ql < nq; ++ql) acc += sh.part[ql][threadIdx.x];
         __syncthreads();
     }
     pdl_wait();   // returns at once after the wait above; covers an empty subset
     const int ix = x0 + (threadIdx.x % kTile);
     const int iy = y0 + (threadIdx.x / kTile);
-    if (ix < a.nx && iy < a.ny) {
+    if ((NT == kTile * kTile || threadIdx.x < kTile * kTile) && ix < a.nx && iy < a.ny) {
         const int n = iy * a.nx + ix;
         apply_epilogue<EPI, TQ, GENPOT>(a, t, n, n, ix, iy, 0, acc);
     }
 }
 
-inline size_t run_smem_bytes() { return sizeof(RunShared); }
+template <int NT>
+constexpr size_t run_smem_bytes() {
+    return sizeof(RunShared<kRunViews<NT>>);
+}
 inline size_t tile_smem_bytes() { return sizeof(TileShared); }
 
 // Member update of one tile: the member's algorithm and table type select
