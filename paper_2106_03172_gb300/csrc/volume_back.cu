@@ -105,9 +105,10 @@ __global__ void __launch_bounds__(kBlock) back_slim_kernel(const BackArgs a) {
 // the subset's views among them (a.cands per view), evaluate each one's band
 // piece once for all slices, and leave the nonzero weights, in view and bin
 // order, in shared memory; the warp then walks that list in order
-// (deterministic), and each lane applies the update to its own slices.  Bound by instruction issue.  47 slices of 128^2 (ncu), against 4
-// pixels x 8 z-lanes (back_slim_kernel's layout): anchor of 14 subsets 290 -> 231
-// us, an update 37.5 -> 32.1 us; 24 slices of 96^2, a run call 723 -> 440 us.
+// (deterministic), and each lane applies the update to its own slices.  Bound
+// by instruction issue.  47 slices of 128^2 (ncu), against 4 pixels x 8 z-lanes
+// (back_slim_kernel's layout): anchor of 14 subsets 291 -> 230 us, an update
+// 38 -> 30 us.
 constexpr int kStackPieces = 96;     // list entries per warp (a round adds up to 32)
 
 template <int EPI, typename TQ, bool GENPOT, int W>
