@@ -389,7 +389,7 @@ pet_status pet_plan_create(const pet_geometry *g, const pet_subsets *sub, pet_pl
     if (g->nx < 1 || g->ny < 1 || g->nz < 1 || g->n_angles < 1 || g->n_bins < 1)
         return set_error(PET_ERR_INVALID, "geometry sizes must be >= 1");
     if (g->nx > 16384 || g->ny > 16384) return set_error(PET_ERR_INVALID, "nx, ny must be <= 16384");
-    if (g->n_angles > 1024) return set_error(PET_ERR_INVALID, "n_angles must be <= 1024");
+    if (g->n_angles > kMaxViews) return set_error(PET_ERR_INVALID, "n_angles must be <= 1024");
     if (!(g->pixel_mm > 0.0) || !std::isfinite(g->pixel_mm) || !std::isfinite(g->bin_mm))
         return set_error(PET_ERR_INVALID, "pixel_mm must be positive and finite");
     if (sub->scheme != 0) return set_error(PET_ERR_INVALID, "only the interleaved subset scheme (0) exists");

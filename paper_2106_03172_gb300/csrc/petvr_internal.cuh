@@ -44,6 +44,8 @@ namespace petvr {
 // value and its FP64 rounding residual), and u - ui is evaluated as
 // uf + kc (du + du_lo), whose magnitude stays small exactly when |du| is.
 // ---------------------------------------------------------------------------
+constexpr int kMaxViews = 1024;   // most views of a plan
+
 struct alignas(16) ViewParams {
     float du;     // minor displacement (pixels) per major step (FP32 value)
     float du_lo;  // FP64 residual du_exact - du
@@ -261,6 +263,27 @@ cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, s
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
+// Shared memory of a block beyond 48 KB (static and dynamic) has to be allowed,
+// kernel by kernel.  The allowance is the kernel's, shared by all of its launches:
+// it is raised once per kernel and device, to `most`, the largest amount any
+// launch of that kernel may ask for, so that host threads launching it at the
+// same time, and graphs captured before, never find it lower than their own.
+template <auto kKernel>
+cudaError_t allow_shared_memory(size_t most) {
+    static std::atomic<uint64_t> raised{0};          // a bit per device
+    int device = 0;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e != cudaSuccess) return e;
+    const uint64_t bit = device < 64 ? uint64_t(1) << device : 0;
+    if (raised.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute((const void *)kKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    if (e == cudaSuccess)
+        raised.fetch_or(bit, std::memory_order_release);
+    else
+        cudaGetLastError();                          // not the next launch's error
+    return e;
 }
 
 // ---------------------------------------------------------------------------

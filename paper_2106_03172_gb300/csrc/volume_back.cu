@@ -359,22 +359,32 @@ struct VolumeBack {
     cudaStream_t s;
     int max_views;
 
+    // Launch with the views of the largest subset staged in shared memory.  Beside
+    // the kernels' own at most kOwnShared bytes, 48 KB hold 787 views of them.
+    template <auto kKernel>
+    pet_status launch(dim3 grid) const {
+        constexpr size_t kPerView = sizeof(ViewParams) + sizeof(int), kOwnShared = 8 << 10;
+        const size_t smem = (size_t)max_views * kPerView;
+        if (smem + kOwnShared > (48 << 10)) {
+            const cudaError_t e = allow_shared_memory<kKernel>(kMaxViews * kPerView);
+            if (e != cudaSuccess)
+                return set_error(PET_ERR_CUDA, std::string("volume back projection: ") + cudaGetErrorString(e));
+        }
+        kKernel<<<grid, kBlock, smem, s>>>(a);
+        return check_launch("volume back projection");
+    }
+
     template <int EPI, typename TQ, bool GENPOT>
     pet_status run() const {
-        const size_t smem = (size_t)max_views * (sizeof(ViewParams) + sizeof(int));
         if (a.axial && a.nz <= 8) {                     // multi-ring, layers in registers
             const dim3 grid((unsigned)((a.nx * a.ny + kColumns - 1) / kColumns), (unsigned)ny_grid);
-            if (a.nz <= 4)
-                ring_back_column_kernel<EPI, TQ, GENPOT, 4><<<grid, kBlock, smem, s>>>(a);
-            else
-                ring_back_column_kernel<EPI, TQ, GENPOT, 8><<<grid, kBlock, smem, s>>>(a);
-            return check_launch("ring_back_column_kernel");
+            return a.nz <= 4 ? launch<ring_back_column_kernel<EPI, TQ, GENPOT, 4>>(grid)
+                             : launch<ring_back_column_kernel<EPI, TQ, GENPOT, 8>>(grid);
         }
         if (a.axial) {                                  // multi-ring, one voxel per lane group
             const long long threads = (long long)a.nx * a.ny * a.nz * kLanes;
             const dim3 grid((unsigned)((threads + kBlock - 1) / kBlock), (unsigned)ny_grid);
-            ring_back_kernel<EPI, TQ, GENPOT><<<grid, kBlock, smem, s>>>(a);
-            return check_launch("ring_back_kernel");
+            return launch<ring_back_kernel<EPI, TQ, GENPOT>>(grid);
         }
         const int w = stack_lane_slices(a.nz);
         const long long pixels = (long long)a.nx * a.ny;
@@ -382,11 +392,10 @@ struct VolumeBack {
         const long long warps = w == 0 ? (pixels + kStackPixels - 1) / kStackPixels : pixels * stack_windows(a.nz);
         const dim3 grid((unsigned)((warps + kBlock / 32 - 1) / (kBlock / 32)), (unsigned)ny_grid);
         switch (w) {
-            case 0: back_slim_kernel<EPI, TQ, GENPOT, kSlimSlices / 8><<<grid, kBlock, smem, s>>>(a); break;
-            case 1: back_stack_kernel<EPI, TQ, GENPOT, 1><<<grid, kBlock, smem, s>>>(a); break;
-            default: back_stack_kernel<EPI, TQ, GENPOT, 2><<<grid, kBlock, smem, s>>>(a); break;
+            case 0: return launch<back_slim_kernel<EPI, TQ, GENPOT, kSlimSlices / 8>>(grid);
+            case 1: return launch<back_stack_kernel<EPI, TQ, GENPOT, 1>>(grid);
+            default: return launch<back_stack_kernel<EPI, TQ, GENPOT, 2>>(grid);
         }
-        return check_launch("back_stack_kernel");
     }
 };
 
