@@ -145,17 +145,14 @@ __global__ void __launch_bounds__(kBlock, kBackMinBlocks)
 // bound was faster alone and slower with several streams.  256^2: a SAGA epoch
 // 160 us (no bound: 176), the four-method step on four streams 2055 us (1994);
 // at an even share of three and more the register limit does.
-size_t residency_smem(const void *kernel, int blocks, size_t base) {
-    const int cap = (blocks + sm_count() - 1) / sm_count() + 1;
+// The kernel's allowance is the amount of the tightest bound, whatever this launch asks for.
+template <auto kKernel>
+size_t residency_smem(int blocks, size_t base) {
+    const int cap = (blocks + sm_count() - 1) / sm_count() + 1;      // 2 and more
     if (cap > 3) return base;
-    constexpr size_t kPerSm = 227 << 10, kReserved = 1 << 10;     // shared memory of an SM; a block's own overhead
-    const size_t need = kPerSm / (size_t)(cap + 1) - kReserved + 1024;
-    if (need <= base ||
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need) != cudaSuccess) {
-        cudaGetLastError();
-        return base;
-    }
-    return need;
+    constexpr size_t kPerSm = 227 << 10;                             // shared memory of an SM
+    const size_t need = kPerSm / (size_t)(cap + 1);
+    return need > base && allow_shared_memory<kKernel>(kPerSm / 3) == cudaSuccess ? need : base;
 }
 
 // Single-slice back-projection launch of one epilogue / table type / potential.
@@ -190,9 +187,9 @@ struct TileBack {
                 return run_launch<EPI, TQ, GENPOT, 1024>(grid);
             return run_launch<EPI, TQ, GENPOT, 512>(grid);
         }
-        const auto k = back_tile_kernel<EPI, TQ, GENPOT>;
+        constexpr auto k = back_tile_kernel<EPI, TQ, GENPOT>;
         const size_t smem = tile_smem_bytes();
-        launch_dependent(k, grid, dim3(kBlock), a.t_dev ? residency_smem((const void *)k, tiles, smem) : smem, s, a);
+        launch_dependent(k, grid, dim3(kBlock), a.t_dev ? residency_smem<k>(tiles, smem) : smem, s, a);
         return check_launch("back_tile_kernel");
     }
 };
