@@ -289,7 +289,7 @@ __device__ __forceinline__ void stage_bins(int nq, int bw, Load &&load) {
 template <int EPI, typename TQ, bool GENPOT, bool COH = false>
 __device__ __forceinline__ void back_tile_body(const BackArgs &a, const int t, const int bx) {
     constexpr int NT = kTile * kTile;
-    extern __shared__ unsigned char smem_raw[];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     TileShared &sh = *reinterpret_cast<TileShared *>(smem_raw);
     const int vb = __ldg(a.sub_off + t);
     const int nv = __ldg(a.sub_off + t + 1) - vb;
@@ -430,7 +430,7 @@ struct RunShared {
 
 template <int EPI, typename TQ, bool GENPOT, int NT>
 __device__ __forceinline__ void back_run_body(const BackArgs &a, const int t, const int bx) {
-    extern __shared__ unsigned char smem_raw[];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int kViews = kRunViews<NT>;
     RunShared<kViews> &sh = *reinterpret_cast<RunShared<kViews> *>(smem_raw);
     const int vb = __ldg(a.sub_off + t);

@@ -25,7 +25,7 @@ namespace {
 // lane then applies the update to its own slices.
 template <int EPI, typename TQ, bool GENPOT, int ZW>
 __global__ void __launch_bounds__(kBlock) back_slim_kernel(const BackArgs a) {
-    extern __shared__ unsigned char smem_raw[];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     ViewParams *s_views = reinterpret_cast<ViewParams *>(smem_raw);
     const int t = a.t_dev ? __ldg(a.t_dev) : a.t0 + (int)blockIdx.y;
     const int vb = __ldg(a.sub_off + t);
@@ -113,7 +113,7 @@ constexpr int kStackPieces = 96;     // list entries per warp (a round adds up t
 
 template <int EPI, typename TQ, bool GENPOT, int W>
 __global__ void __launch_bounds__(kBlock, 5) back_stack_kernel(const BackArgs a) {
-    extern __shared__ unsigned char smem_raw[];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ float2 s_piece[kBlock / 32][kStackPieces];   // ratio offset, weight
     ViewParams *s_views = reinterpret_cast<ViewParams *>(smem_raw);
     const int t = a.t_dev ? __ldg(a.t_dev) : a.t0 + (int)blockIdx.y;
@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(kBlock, 5) back_stack_kernel(const BackArgs a)
 // piece_zeta / layer_fraction, the forward projector's own expressions).
 template <int EPI, typename TQ, bool GENPOT>
 __global__ void __launch_bounds__(kBlock) ring_back_kernel(const BackArgs a) {
-    extern __shared__ unsigned char smem_raw[];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     ViewParams *s_views = reinterpret_cast<ViewParams *>(smem_raw);
     const int t = a.t_dev ? __ldg(a.t_dev) : a.t0 + (int)blockIdx.y;
     const int vb = __ldg(a.sub_off + t);
@@ -276,7 +276,7 @@ constexpr int kViewLanes = kBlock / kColumns;
 
 template <int EPI, typename TQ, bool GENPOT, int LMAX>
 __global__ void __launch_bounds__(kBlock) ring_back_column_kernel(const BackArgs a) {
-    extern __shared__ unsigned char smem_raw[];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ float s_sum[kViewLanes][LMAX][kColumns];
     ViewParams *s_views = reinterpret_cast<ViewParams *>(smem_raw);
     const int t = a.t_dev ? __ldg(a.t_dev) : a.t0 + (int)blockIdx.y;
