@@ -41,9 +41,19 @@ __global__ void __launch_bounds__(kBlock, kBackMinBlocks) back_tile_kernel(const
     back_tile_body<EPI, TQ, GENPOT>(a, t, blockIdx.x);
 }
 
-template <int EPI, typename TQ, bool GENPOT, int NT = kBlock>
-__global__ void __launch_bounds__(NT) back_run_kernel(const BackArgs a) {
+// Runs: at 48 registers two 512-thread blocks fit an SM, or five of 256.
+constexpr int kRunRegs = 48;
+
+template <int EPI, typename TQ, bool GENPOT, int NT>
+__global__ void __maxnreg__(kRunRegs) back_run_kernel(const BackArgs a) {
     back_run_body<EPI, TQ, GENPOT, NT>(a, a.t0 + (int)blockIdx.y, blockIdx.x);
+}
+
+// Without that bound the compiler takes 40 registers for 512 threads (three blocks
+// an SM) and 57 for 1024 (one).
+template <int NT>
+__global__ void __launch_bounds__(NT) back_run_plain_kernel(const BackArgs a) {
+    back_run_body<EPI_PLAIN, float, false, NT>(a, a.t0 + (int)blockIdx.y, blockIdx.x);
 }
 
 // Persistent batched back projection + update: a resident grid whose blocks
@@ -162,10 +172,30 @@ struct TileBack {
     cudaStream_t s;
     int max_views;
 
-    template <int EPI, typename TQ, bool GENPOT, int NT>
+    template <auto kKernel, int NT>
     pet_status run_launch(dim3 grid) const {
-        launch_dependent(back_run_kernel<EPI, TQ, GENPOT, NT>, grid, dim3(NT), run_smem_bytes<NT>(), s, a);
+        launch_dependent(kKernel, grid, dim3(NT), run_smem_bytes<NT>(), s, a);
         return check_launch("back_run_kernel");
+    }
+
+    // Plain back projections (no update behind them): runs, one per thread and pass.
+    // The blocks of a launch are placed while the kernel ahead still runs, so an SM
+    // that can take three piles them up where two each would do.  Forward + back in
+    // a graph, bins = pixels:
+    // - up to two blocks an SM: 512 threads at 48 registers, 128^2 x 64 views
+    //   18.5 us (40 registers, so three an SM: 24.2), 256^2 x 90 36.3 (44.7);
+    // - one block an SM and several passes: 1024 threads, 128^2 x 90 16.4 (21.5);
+    //   with 256^2's 256 tiles 38.7 (36.3);
+    // - more blocks: 512 threads, three an SM, 300^2 x 30 18.0 (two: 20.7);
+    // - many blocks, few views: 256 threads (a run each), 512^2 x 6 13.9 (15.2);
+    //   300^2's 361 tiles 8.1 (7.4).
+    pet_status run_plain(dim3 grid) const {
+        const int blocks = (int)(grid.x * grid.y), sms = sm_count();
+        if (blocks <= sms && max_views > 64) return run_launch<back_run_plain_kernel<1024>, 1024>(grid);
+        if (blocks <= 2 * sms) return run_launch<back_run_kernel<EPI_PLAIN, float, false, 512>, 512>(grid);
+        if (blocks > 3 * sms && max_views <= 8)
+            return run_launch<back_run_kernel<EPI_PLAIN, float, false, kBlock>, kBlock>(grid);
+        return run_launch<back_run_plain_kernel<512>, 512>(grid);
     }
 
     template <int EPI, typename TQ, bool GENPOT>
@@ -173,20 +203,8 @@ struct TileBack {
         const int tiles = ((a.nx + kTile - 1) / kTile) * ((a.ny + kTile - 1) / kTile);
         const dim3 grid((unsigned)tiles, (unsigned)ny_grid);
         if constexpr (EPI == EPI_ANCHOR || EPI == EPI_SAGA_INIT || EPI == EPI_SAGAEM_INIT)
-            return run_launch<EPI, TQ, GENPOT, kBlock>(grid);
-        // Plain back projections (no update behind them): runs, one per thread and
-        // pass.  Forward + back, 512 threads against staged bins (bins = pixels):
-        // 300^2 x 270 views 131.9 us (140.5), 300^2 x 30 18.6 (18.2), 477x461 x 30
-        // 33.5 (30.1), 512^2 x 500 648 (581); bins of 2/3 of a pixel 182 (225),
-        // 24.6 (29.2), 45.7 (47.0), 885 (896).  Where at most two blocks share an
-        // SM and there are several passes, 1024 threads: 213x199 x 220 views
-        // 72.7 us (512 threads 89.8, staged bins 92.5); with 300^2 x 270's 361
-        // tiles 139.9 (512: 131.9), with 28 views 15.8 (15.6).
-        if constexpr (EPI == EPI_PLAIN) {
-            if (tiles * ny_grid <= 2 * sm_count() && max_views > 2 * kRunViews<1024>)
-                return run_launch<EPI, TQ, GENPOT, 1024>(grid);
-            return run_launch<EPI, TQ, GENPOT, 512>(grid);
-        }
+            return run_launch<back_run_kernel<EPI, TQ, GENPOT, kBlock>, kBlock>(grid);
+        if constexpr (EPI == EPI_PLAIN) return run_plain(grid);
         constexpr auto k = back_tile_kernel<EPI, TQ, GENPOT>;
         const size_t smem = tile_smem_bytes();
         launch_dependent(k, grid, dim3(kBlock), a.t_dev ? residency_smem<k>(tiles, smem) : smem, s, a);
