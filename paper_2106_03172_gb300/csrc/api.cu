@@ -165,6 +165,7 @@ BackArgs back_args(const pet_plan *pl, const float *r, int subset, bool natural)
     a.sens = pl->d_sens;
     a.bw = pl->bw;
     a.cand = pl->cand;
+    a.fineness = pl->fineness;
     a.cands = pl->cands;
     a.cand_rounds = pl->cand_rounds;
     return a;
@@ -424,6 +425,7 @@ pet_status pet_plan_create(const pet_geometry *g, const pet_subsets *sub, pet_pl
     pl->nb = g->n_bins;
     bins_division(pl->nb, pl->nb_mul, pl->nb_shift);
     tile_bins(g->pixel_mm, ds_chk, pl->nb, pl->nx, pl->ny, pl->bw, pl->cand);
+    pl->fineness = (float)(g->pixel_mm / ds_chk);
     stack_candidates(g->pixel_mm, ds_chk, pl->nb, pl->nx, pl->ny, pl->cands, pl->cand_rounds);
     pl->ns = sub->n_subsets;
     pl->N = (int)N;

@@ -46,7 +46,8 @@ constexpr int kRunRegs = 48;
 
 template <int EPI, typename TQ, bool GENPOT, int NT>
 __global__ void __maxnreg__(kRunRegs) back_run_kernel(const BackArgs a) {
-    back_run_body<EPI, TQ, GENPOT, NT>(a, a.t0 + (int)blockIdx.y, blockIdx.x);
+    const int t = a.t_dev ? __ldg(a.t_dev) : a.t0 + (int)blockIdx.y;
+    back_run_body<EPI, TQ, GENPOT, NT>(a, t, blockIdx.x);
 }
 
 // Without that bound the compiler takes 40 registers for 512 threads (three blocks
@@ -165,6 +166,48 @@ size_t residency_smem(int blocks, size_t base) {
     return need > base && allow_shared_memory<kKernel>(kPerSm / 3) == cudaSuccess ? need : base;
 }
 
+// Whether an update from `views` views over `tiles` tiles takes runs instead of
+// staged bins (the same bits).  A thread of the staged bins reads two or three
+// candidates a view in an unrolled loop, however wide the bins, and more of them in
+// a loop of its own; a run evaluates each band it meets once, in a longer chain, and
+// 16 views at a time.  us per SAGA update in a graph, staged bins (runs):
+// - up to two tiles an SM: 512 threads.  More than three candidates: 64^2 at 4 bins a
+//   pixel x 5 views 7.3 (8.0), x 6 8.4 (7.9), x 16 17.2 (11.0); 128^2 at 2.2 x 9 9.3
+//   (9.7), x 14 12.4 (10.2).  Three: 48^2 at 1.54 bins a pixel x 10 6.2 (5.6), 256^2
+//   x 14 12.3 (11.1), x 20 17.3 (15.7); at 2, 128^2 x 20 10.9 (13.0).  Two: a bin a
+//   pixel 128^2 x 14 6.7 (7.0), x 60 16.8 (18.8); two tiles an SM, 256^2 x 9 8.1
+//   (9.2), x 12 9.1 (9.5), x 14 10.0 (8.8), x 20 11.5 (11.9), x 32 17.3 (15.7);
+//   wider bins, of which a run meets fewer: 201x199 at 0.6 x 14 8.2 (6.8).
+// - up to four: a thread a run.  300^2 at 2.2 x 12 20.2 (16.1), at 4 x 16 38.2 (39.4);
+//   350^2 at 1 x 6 8.8 (10.1).
+// - beyond: 256 threads.  Few views 512^2 x 4 14.0 (12.0), x 2 10.0 (10.6); wider bins
+//   800x700 at 0.6 x 8 31.4 (24.4); four or five candidates 400^2 at 2.2 x 8 21.2
+//   (18.2); more, 400^2 at 12 x 8 57.5 (64.7).
+// 1444 points against runs everywhere with a thread each: 0.88 of the time on
+// average (staged bins everywhere 0.93, and a quarter of the points slower).
+bool update_by_runs(const BackArgs &a, int tiles, int views) {
+    const int sms = sm_count();
+    const bool wide_bins = a.fineness < 0.9f;
+    if (tiles > 4 * sms)
+        return a.cand <= 2 ? wide_bins || (views > 2 && views <= 6) : a.cand == 4 || a.cand == 5;
+    constexpr int kPass = kRunViews<512>, kNever = kMaxViews;
+    const int passes = (views + kPass - 1) / kPass;
+    if (tiles > 2 * sms) return a.cand > 3 && a.fineness < 3.0f && views > 8 * passes;
+    int most = kNever;                                      // views up to which staged bins are faster
+    const bool few = tiles <= sms / 8;
+    if (a.cand > 3)
+        most = (few ? 5 : 8) * passes;
+    else if (a.cand == 3 && a.fineness < 1.8f)
+        most = tiles > sms ? 12 : (few ? 9 : 12) * passes;
+    else if (a.cand == 3)
+        most = few ? 15 * passes : kNever;
+    else if (wide_bins)
+        most = (tiles > sms ? 8 : 10) * passes;
+    else if (tiles > sms)
+        most = 12 * passes;
+    return views > most;
+}
+
 // Single-slice back-projection launch of one epilogue / table type / potential.
 struct TileBack {
     const BackArgs &a;
@@ -173,8 +216,8 @@ struct TileBack {
     int max_views;
 
     template <auto kKernel, int NT>
-    pet_status run_launch(dim3 grid) const {
-        launch_dependent(kKernel, grid, dim3(NT), run_smem_bytes<NT>(), s, a);
+    pet_status run_launch(dim3 grid, int threads = NT) const {
+        launch_dependent(kKernel, grid, dim3((unsigned)threads), run_smem_bytes<NT>(), s, a);
         return check_launch("back_run_kernel");
     }
 
@@ -202,13 +245,22 @@ struct TileBack {
     pet_status run() const {
         const int tiles = ((a.nx + kTile - 1) / kTile) * ((a.ny + kTile - 1) / kTile);
         const dim3 grid((unsigned)tiles, (unsigned)ny_grid);
-        if constexpr (EPI == EPI_ANCHOR || EPI == EPI_SAGA_INIT || EPI == EPI_SAGAEM_INIT)
+        if constexpr (EPI == EPI_PLAIN) {
+            return run_plain(grid);
+        } else if constexpr (EPI == EPI_ANCHOR || EPI == EPI_SAGA_INIT || EPI == EPI_SAGAEM_INIT) {
             return run_launch<back_run_kernel<EPI, TQ, GENPOT, kBlock>, kBlock>(grid);
-        if constexpr (EPI == EPI_PLAIN) return run_plain(grid);
-        constexpr auto k = back_tile_kernel<EPI, TQ, GENPOT>;
-        const size_t smem = tile_smem_bytes();
-        launch_dependent(k, grid, dim3(kBlock), a.t_dev ? residency_smem<k>(tiles, smem) : smem, s, a);
-        return check_launch("back_tile_kernel");
+        } else {
+            if (update_by_runs(a, tiles, max_views)) {
+                const int sms = sm_count();
+                if (tiles <= 2 * sms) return run_launch<back_run_kernel<EPI, TQ, GENPOT, 512>, 512>(grid);
+                return run_launch<back_run_kernel<EPI, TQ, GENPOT, 0>, 0>(
+                    grid, tiles > 4 * sms ? kBlock : std::max(kBlock, 32 * std::min(max_views, kRunViews<0>)));
+            }
+            constexpr auto k = back_tile_kernel<EPI, TQ, GENPOT>;
+            const size_t smem = tile_smem_bytes();
+            launch_dependent(k, grid, dim3(kBlock), a.t_dev ? residency_smem<k>(tiles, smem) : smem, s, a);
+            return check_launch("back_tile_kernel");
+        }
     }
 };
 

@@ -416,8 +416,8 @@ __device__ __forceinline__ void back_tile_body(const BackArgs &a, const int t, c
 // and 35.3M (ncu).
 constexpr int kRun = 8;
 
-// Views per shared-memory pass of an NT-thread block: a run per thread at 512
-// threads and more, two per thread at 256.
+// Views per shared-memory pass of an NT-thread block (0: as many threads as the
+// launch has): a run per thread at 512 threads and more, two per thread at 256.
 template <int NT>
 constexpr int kRunViews = NT > 512 ? NT / 32 : 16;
 
@@ -436,7 +436,7 @@ __device__ __forceinline__ void back_run_body(const BackArgs &a, const int t, co
     const int vb = __ldg(a.sub_off + t);
     const int nv = __ldg(a.sub_off + t + 1) - vb;
     const int r_view0 = a.t_dev ? vb : a.r_view0;
-    constexpr int nthr = NT;                      // >= kTile * kTile
+    const int nthr = NT ? NT : blockDim.x;        // >= kTile * kTile
 
     const int tiles_x = (a.nx + kTile - 1) / kTile;
     const int x0 = (bx % tiles_x) * kTile;

@@ -387,6 +387,7 @@ struct BackArgs {
     int r_view0;          // view position of r[0] (ignored when t_dev is set: r is
                           //   then the compact ratio of subset *t_dev)
     int bw, cand;         // single-slice tile kernel: bins staged per view, most candidates of a pixel
+    float fineness;       // bins per pixel width
     int nx, ny, nz, nb, ns;  // nz: image entries per pixel (slices, or layers when axial)
     int axial;            // multi-ring: layers are coupled (6-neighbourhood penalty) and the
                           //   sensitivities are per voxel ([ns][nx*ny*nz]); else per pixel
@@ -540,6 +541,7 @@ struct pet_plan {
     int fwd_chunks = 0;             // single-slice forward: band chunks per ray (8, 16 or 32)
     int back_run = 8;               // the caller's choice (4 or 8); no launch shape depends on it
     int bw = 0, cand = 0;           // single-slice back projection (BackArgs)
+    float fineness = 1.0f;
     int cands = 1, cand_rounds = 1;     // slice stacks (BackArgs)
     unsigned nb_mul = 0;            // division of a ray index by nb (bins_division)
     int nb_shift = 0;
