@@ -1816,6 +1816,7 @@ void fill_member(BatchMember &m, const pet_state *st, float alpha, const int *se
     m.nb_shift = pl->nb_shift;
     m.bw = pl->bw;
     m.cand = pl->cand;
+    m.runs = batch_runs(pl) ? 1 : 0;
     m.ns = pl->ns;
     m.sens_t = pl->d_sens_t;
     m.sens = pl->d_sens;
@@ -2023,6 +2024,13 @@ void build_batch_dataflow(pet_batch *b, int n_iter, const std::vector<std::vecto
         }
 }
 
+// Whether some member of the batch takes runs.
+bool any_runs(const pet_batch *b) {
+    for (const pet_state *st : b->states)
+        if (batch_runs(st->prob->plan)) return true;
+    return false;
+}
+
 // The dependency-driven epoch on stream s: the iterate copy (odd update
 // counts), SEM statistics due, the counters' reset, then one launch.
 pet_status enqueue_batch_dataflow(pet_batch *b, int32_t n_iter, bool genpot, cudaStream_t s) {
@@ -2042,7 +2050,7 @@ pet_status enqueue_batch_dataflow(pet_batch *b, int32_t n_iter, bool genpot, cud
     const DfSeg &last = b->h_df.back();
     PET_TRY(launch_zero_ints(b->d_df_done, n_segs + 1, s));
     return launch_dataflow_epoch(b->d_members, b->d_df, n_segs, last.first + last.count, odd ? 1 : 0, b->d_df_done,
-                                 b->d_status, b->wait_limit, genpot, s);
+                                 b->d_status, b->wait_limit, genpot, any_runs(b), s);
 }
 
 // All launches of one batched epoch on stream s (phases from build_batch_phases).
@@ -2072,7 +2080,7 @@ pet_status enqueue_batch_epoch(pet_batch *b, int32_t n_iter, const std::vector<s
                                                   in_is_img ? 1 : 0, b->d_claims + ph.claim, false, s));
             } else if (ph.kind == 1) {
                 PET_TRY(launch_persistent_back(b->d_members, b->d_segs + ph.seg_off, ph.n_segs, ph.n_items, i,
-                                               in_is_img ? 1 : 0, b->d_claims + ph.claim, ph.genpot != 0, s));
+                                               in_is_img ? 1 : 0, b->d_claims + ph.claim, ph.genpot != 0, any_runs(b), s));
             } else {
                 for (int j = 0; j < n; ++j) {
                     if (!anchors[j][i]) continue;

@@ -60,18 +60,20 @@ __global__ void __launch_bounds__(NT) back_run_plain_kernel(const BackArgs a) {
 // Persistent batched back projection + update: a resident grid whose blocks
 // claim work items until the list is exhausted.  An item is one tile of a
 // member's update (WK_BACK_UPDATE) or one (subset, tile) of a member's anchor
-// back projection (WK_BACK_ANCHOR), run by the same body as the member's own
-// launches, so results are bit-identical to them.
+// back projection (WK_BACK_ANCHOR), by runs or staged bins, with the bits of the
+// member's own launches.
 // Thread 0 claims the item and writes its arguments to shared memory; the
 // segment table is staged in shared memory once per block.
 // GENPOT: the members of this launch use an edge-preserving potential.
-template <bool GENPOT>
+// RUNS: some member's bins are wide enough for runs (batch_runs); a kernel without
+// them is 1 to 3% faster for the others.
+template <bool GENPOT, bool RUNS>
 __global__ void __launch_bounds__(kBlock, kBackMinBlocks)
     persistent_back_kernel(const BatchMember *ms, const WorkSeg *segs, int n_segs, int n_items, int iter,
                            int in_is_img, int *claim) {
     __shared__ WorkSeg s_segs[kSegSmem];
     __shared__ BackArgs s_b;
-    __shared__ int s_item, s_t, s_tile, s_kind, s_algo, s_tq;
+    __shared__ int s_item, s_t, s_tile, s_kind, s_algo, s_tq, s_runs;
     for (int i = threadIdx.x; i < n_segs && i < kSegSmem; i += blockDim.x) s_segs[i] = segs[i];
     const WorkSeg *tab = n_segs <= kSegSmem ? s_segs : segs;
     // the segment table and member descriptors were copied in before the
@@ -136,15 +138,16 @@ __global__ void __launch_bounds__(kBlock, kBackMinBlocks)
                 s_kind = sg.kind;
                 s_algo = m.algo;
                 s_tq = m.table_dtype;
+                s_runs = m.runs;
             }
         }
         __syncthreads();
         if (s_item >= n_items) break;
         const int t = s_t, tile = s_tile;
         if (s_kind == WK_BACK_ANCHOR)
-            back_tile_body<EPI_ANCHOR, float, false>(s_b, t, tile);
+            member_tile<EPI_ANCHOR, float, false, RUNS, false>(s_runs, s_b, t, tile);
         else
-            member_update_tile<GENPOT>(s_algo, s_tq, s_b, t, tile);
+            member_update_tile<GENPOT, RUNS>(s_algo, s_tq, s_runs, s_b, t, tile);
     }
 }
 
@@ -176,8 +179,9 @@ size_t residency_smem(int blocks, size_t base) {
 //   (9.7), x 14 12.4 (10.2).  Three: 48^2 at 1.54 bins a pixel x 10 6.2 (5.6), 256^2
 //   x 14 12.3 (11.1), x 20 17.3 (15.7); at 2, 128^2 x 20 10.9 (13.0).  Two: a bin a
 //   pixel 128^2 x 14 6.7 (7.0), x 60 16.8 (18.8); two tiles an SM, 256^2 x 9 8.1
-//   (9.2), x 12 9.1 (9.5), x 14 10.0 (8.8), x 20 11.5 (11.9), x 32 17.3 (15.7);
-//   wider bins, of which a run meets fewer: 201x199 at 0.6 x 14 8.2 (6.8).
+//   (9.2), x 12 9.1 (9.5), x 14 10.0 (8.8), x 20 11.5 (11.9), x 32 17.3 (15.7), x 60
+//   25.8 (25.7; beside other streams the staged bins are 3% faster); wider bins, of
+//   which a run meets fewer: 201x199 at 0.6 x 14 8.2 (6.8).
 // - up to four: a thread a run.  300^2 at 2.2 x 12 20.2 (16.1), at 4 x 16 38.2 (39.4);
 //   350^2 at 1 x 6 8.8 (10.1).
 // - beyond: 256 threads.  Few views 512^2 x 4 14.0 (12.0), x 2 10.0 (10.6); wider bins
@@ -204,7 +208,7 @@ bool update_by_runs(const BackArgs &a, int tiles, int views) {
     else if (wide_bins)
         most = (tiles > sms ? 8 : 10) * passes;
     else if (tiles > sms)
-        most = 12 * passes;
+        most = passes <= 2 ? 12 * passes : kNever;
     return views > most;
 }
 
@@ -283,14 +287,24 @@ void tile_bins(double pixel_mm, double bin_mm, int nb, int nx, int ny, int &bw, 
     bw = std::min(kStageBins + 1, (int)std::ceil((kTile - 1) * 1.41422 * ratio) + cand + 4);
 }
 
+// Members of a batch fill the grid and are bound by issue: those whose bins are wider
+// than a pixel, of which a run meets fewer, take runs.  Epoch of 5 updates from 8
+// views each, 64 SAGA members of 64^2 to 200^2, us with staged bins (runs): 0.6 bins a
+// pixel 457 (405), 0.77 483 (447), 1.0 524 (503); 24 members of 64^2 to 256^2 with 5
+// to 60 views at 1.0, 12 updates 1630 (1758).  In one dependency-driven launch: 0.6
+// 532 (498), 0.77 581 (559), 1.0 647 (642), and 2106 (2209).
+bool batch_runs(const pet_plan *pl) { return pl->fineness < 0.9f; }
+
 pet_status launch_persistent_back(const BatchMember *d_members, const WorkSeg *d_segs, int n_segs, int n_items,
-                                  int iter, int in_is_img, int *claim, bool general_potential, cudaStream_t s) {
+                                  int iter, int in_is_img, int *claim, bool general_potential, bool runs,
+                                  cudaStream_t s) {
     if (n_items <= 0) return PET_OK;
     void (*k)(const BatchMember *, const WorkSeg *, int, int, int, int, int *) =
-        general_potential ? persistent_back_kernel<true> : persistent_back_kernel<false>;
+        runs ? (general_potential ? persistent_back_kernel<true, true> : persistent_back_kernel<false, true>)
+             : (general_potential ? persistent_back_kernel<true, false> : persistent_back_kernel<false, false>);
     const size_t smem = tile_smem_bytes();
-    static int resident[2] = {};   // blocks per SM by potential class
-    int &per_sm = resident[general_potential ? 1 : 0];
+    static int resident[4] = {};   // blocks per SM of each kernel
+    int &per_sm = resident[(general_potential ? 1 : 0) + (runs ? 2 : 0)];
     if (per_sm == 0 &&
         (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)k, kBlock, smem) != cudaSuccess ||
          per_sm < 1))

@@ -428,7 +428,7 @@ struct RunShared {
     int vid[VIEWS];
 };
 
-template <int EPI, typename TQ, bool GENPOT, int NT>
+template <int EPI, typename TQ, bool GENPOT, int NT, bool COH = false>
 __device__ __forceinline__ void back_run_body(const BackArgs &a, const int t, const int bx) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int kViews = kRunViews<NT>;
@@ -490,7 +490,7 @@ __device__ __forceinline__ void back_run_body(const BackArgs &a, const int t, co
                 float w0, w1;
                 const float tl = band_weights(vp.L, vp.Lm, fminf(e0, e1), fmaxf(e0, e1), w0, w1);
                 const int c = (int)(__float_as_uint(tl) - kRoundBits) + (int)u.x - m0rel;
-                const float r = __ldg(rv + j);
+                const float r = ld_data<COH>(rv + j);
                 if ((unsigned)c < (unsigned)mlen) pp[c * lstep] += w0 * r;
                 if (w1 > 0.0f && (unsigned)(c + 1) < (unsigned)mlen) pp[(c + 1) * lstep] += w1 * r;
             }
@@ -505,7 +505,7 @@ __device__ __forceinline__ void back_run_body(const BackArgs &a, const int t, co
     const int iy = y0 + (threadIdx.x / kTile);
     if ((NT == kTile * kTile || threadIdx.x < kTile * kTile) && ix < a.nx && iy < a.ny) {
         const int n = iy * a.nx + ix;
-        apply_epilogue<EPI, TQ, GENPOT>(a, t, n, n, ix, iy, 0, acc);
+        apply_epilogue<EPI, TQ, GENPOT, COH>(a, t, n, n, ix, iy, 0, acc);
     }
 }
 
@@ -515,23 +515,34 @@ constexpr size_t run_smem_bytes() {
 }
 inline size_t tile_smem_bytes() { return sizeof(TileShared); }
 
+// One tile of a batch member (256 threads), by runs (RUNS: a kernel that has them)
+// or staged bins, the same bits.
+template <int EPI, typename TQ, bool GENPOT, bool RUNS, bool COH>
+__device__ __forceinline__ void member_tile(bool runs, const BackArgs &b, int t, int tile) {
+    if (RUNS && runs)
+        back_run_body<EPI, TQ, GENPOT, kBlock, COH>(b, t, tile);
+    else
+        back_tile_body<EPI, TQ, GENPOT, COH>(b, t, tile);
+}
+
 // Member update of one tile: the member's algorithm and table type select
 // the epilogue (the single-state launch's template arguments).
-template <bool GENPOT, bool COH = false>
-__device__ __forceinline__ void member_update_tile(int algo, int table_dtype, const BackArgs &b, int t, int tile) {
+template <bool GENPOT, bool RUNS, bool COH = false>
+__device__ __forceinline__ void member_update_tile(int algo, int table_dtype, bool runs, const BackArgs &b, int t,
+                                                   int tile) {
     switch (algo) {
-        case PET_ALGO_OSEM: back_tile_body<EPI_OSEM, float, GENPOT, COH>(b, t, tile); break;
-        case PET_ALGO_SVREM: back_tile_body<EPI_SVREM, float, GENPOT, COH>(b, t, tile); break;
+        case PET_ALGO_OSEM: member_tile<EPI_OSEM, float, GENPOT, RUNS, COH>(runs, b, t, tile); break;
+        case PET_ALGO_SVREM: member_tile<EPI_SVREM, float, GENPOT, RUNS, COH>(runs, b, t, tile); break;
         case PET_ALGO_SAGA:
             if (table_dtype == PET_TABLE_BF16)
-                back_tile_body<EPI_SAGA, __nv_bfloat16, GENPOT, COH>(b, t, tile);
+                member_tile<EPI_SAGA, __nv_bfloat16, GENPOT, RUNS, COH>(runs, b, t, tile);
             else
-                back_tile_body<EPI_SAGA, float, GENPOT, COH>(b, t, tile);
+                member_tile<EPI_SAGA, float, GENPOT, RUNS, COH>(runs, b, t, tile);
             break;
-        case PET_ALGO_SGA: back_tile_body<EPI_SGA, float, GENPOT, COH>(b, t, tile); break;
-        case PET_ALGO_SEM: back_tile_body<EPI_SEM, float, GENPOT, COH>(b, t, tile); break;
-        case PET_ALGO_SAGAEM: back_tile_body<EPI_SAGAEM, float, GENPOT, COH>(b, t, tile); break;
-        default: back_tile_body<EPI_SVRG, float, GENPOT, COH>(b, t, tile); break;
+        case PET_ALGO_SGA: member_tile<EPI_SGA, float, GENPOT, RUNS, COH>(runs, b, t, tile); break;
+        case PET_ALGO_SEM: member_tile<EPI_SEM, float, GENPOT, RUNS, COH>(runs, b, t, tile); break;
+        case PET_ALGO_SAGAEM: member_tile<EPI_SAGAEM, float, GENPOT, RUNS, COH>(runs, b, t, tile); break;
+        default: member_tile<EPI_SVRG, float, GENPOT, RUNS, COH>(runs, b, t, tile); break;
     }
 }
 

@@ -25,10 +25,9 @@
 // launch (iterates, ratios, anchor caches) are read with plain loads (the
 // bodies' COH variant), not through the read-only data path.
 //
-// An item is one block of the member's own single-state launch, run by the
-// same body with the same launch shape, so each member's results are
-// bit-identical to its own epoch calls (the finish items repeat the finish
-// kernels' arithmetic).
+// An item is one block of the member's own single-state launch, with the same
+// weights and order of sums, so each member's results are bit-identical to its
+// own epoch calls (the finish items repeat the finish kernels' arithmetic).
 #include <algorithm>
 
 #include "bodies.cuh"
@@ -93,7 +92,8 @@ __device__ __forceinline__ void finish_pixel(const FinArgs &a, long long i) {
     }
 }
 
-template <bool GENPOT>
+// RUNS: some member takes runs (batch_runs).
+template <bool GENPOT, bool RUNS>
 __global__ void __maxnreg__(kDataflowRegs)
     dataflow_epoch_kernel(const BatchMember *ms, const DfSeg *segs, int n_segs, int n_items, int odd, int *done,
                           int *status, long long wait_limit) {
@@ -102,7 +102,7 @@ __global__ void __maxnreg__(kDataflowRegs)
         BackArgs b;
         FinArgs fin;
     } s_args;
-    __shared__ int s_item, s_seg, s_ok, s_kind, s_shape, s_bx, s_t, s_algo, s_tq;
+    __shared__ int s_item, s_seg, s_ok, s_kind, s_shape, s_bx, s_t, s_algo, s_tq, s_runs;
     int *claim = done;             // done[0]: the claim counter; done[1 + k]: items of segment k done
     int *seg_done = done + 1;
     // the counters were zeroed by the kernel ahead of this one
@@ -134,6 +134,7 @@ __global__ void __maxnreg__(kDataflowRegs)
                     s_bx = local;
                     s_algo = m.algo;
                     s_tq = m.table_dtype;
+                    s_runs = m.runs;
                     if (sg.kind == DF_FWD_UPDATE || sg.kind == DF_FWD_ANCHOR) {
                         FwdArgs a{};
                         a.views = m.views;
@@ -232,9 +233,9 @@ __global__ void __maxnreg__(kDataflowRegs)
                 const long long i = (long long)bx * kBlock + threadIdx.x;
                 if (i < s_args.fin.plane) finish_pixel(s_args.fin, i);
             } else if (kind == DF_BACK_ANCHOR) {
-                back_tile_body<EPI_ANCHOR, float, false, true>(s_args.b, s_t, bx);
+                member_tile<EPI_ANCHOR, float, false, RUNS, true>(s_runs, s_args.b, s_t, bx);
             } else {
-                member_update_tile<GENPOT, true>(s_algo, s_tq, s_args.b, s_t, bx);
+                member_update_tile<GENPOT, RUNS, true>(s_algo, s_tq, s_runs, s_args.b, s_t, bx);
             }
         }
         __syncthreads();
@@ -249,13 +250,14 @@ __global__ void __maxnreg__(kDataflowRegs)
 
 pet_status launch_dataflow_epoch(const BatchMember *d_members, const DfSeg *d_segs, int n_segs, int n_items,
                                  int odd, int *d_done, int *d_status, long long wait_limit, bool general_potential,
-                                 cudaStream_t s) {
+                                 bool runs, cudaStream_t s) {
     if (n_items <= 0) return PET_OK;
     void (*k)(const BatchMember *, const DfSeg *, int, int, int, int *, int *, long long) =
-        general_potential ? dataflow_epoch_kernel<true> : dataflow_epoch_kernel<false>;
+        runs ? (general_potential ? dataflow_epoch_kernel<true, true> : dataflow_epoch_kernel<false, true>)
+             : (general_potential ? dataflow_epoch_kernel<true, false> : dataflow_epoch_kernel<false, false>);
     const size_t smem = tile_smem_bytes();
-    static int resident[2] = {};   // blocks per SM by potential class
-    int &per_sm = resident[general_potential ? 1 : 0];
+    static int resident[4] = {};   // blocks per SM of each kernel
+    int &per_sm = resident[(general_potential ? 1 : 0) + (runs ? 2 : 0)];
     if (per_sm == 0 &&
         (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)k, kBlock, smem) != cudaSuccess ||
          per_sm < 1))

@@ -426,6 +426,7 @@ struct BatchMember {
     unsigned nb_mul;       // division by nb (FwdArgs)
     int nb_shift;
     int bw, cand;          // back-projection tiles (BackArgs)
+    int runs;              // its tiles take runs instead of staged bins (batch_runs)
     const float *sens_t;
     const float *sens;
     const float *g;
@@ -698,12 +699,14 @@ pet_status launch_persistent_forward(const BatchMember *d_members, const WorkSeg
                                      int iter, int in_is_img, int *claim, bool objective, cudaStream_t s);
 void tile_bins(double pixel_mm, double bin_mm, int nb, int nx, int ny, int &bw, int &cand);   // BackArgs
 pet_status launch_persistent_back(const BatchMember *d_members, const WorkSeg *d_segs, int n_segs, int n_items,
-                                  int iter, int in_is_img, int *claim, bool general_potential, cudaStream_t s);
+                                  int iter, int in_is_img, int *claim, bool general_potential, bool runs,
+                                  cudaStream_t s);
+bool batch_runs(const pet_plan *pl);   // whether a batch member's tiles take runs
 pet_status launch_zero_ints(int *p, int n, cudaStream_t s);
 // Dependency-driven batched epoch (dataflow.cu): the whole list in one launch.
 pet_status launch_dataflow_epoch(const BatchMember *d_members, const DfSeg *d_segs, int n_segs, int n_items,
                                  int odd, int *d_done, int *d_status, long long wait_limit, bool general_potential,
-                                 cudaStream_t s);
+                                 bool runs, cudaStream_t s);
 int sm_count();
 pet_status launch_batch_objective_finish(const BatchMember *d_members, int n_members, int pen_blocks,
                                          cudaStream_t s);
