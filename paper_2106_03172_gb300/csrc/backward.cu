@@ -50,11 +50,12 @@ __global__ void __maxnreg__(kRunRegs) back_run_kernel(const BackArgs a) {
     back_run_body<EPI, TQ, GENPOT, NT>(a, t, blockIdx.x);
 }
 
-// Without that bound the compiler takes 40 registers for 512 threads (three blocks
-// an SM) and 57 for 1024 (one).
-template <int NT>
-__global__ void __launch_bounds__(NT) back_run_plain_kernel(const BackArgs a) {
-    back_run_body<EPI_PLAIN, float, false, NT>(a, a.t0 + (int)blockIdx.y, blockIdx.x);
+// All-subset launches and plain back projections without that bound: the compiler
+// takes 40 registers for table fills (six blocks of 256 threads an SM; 48 for
+// anchors) and for 512 threads (three an SM), and 57 for 1024 (one).
+template <int EPI, typename TQ, bool GENPOT, int NT>
+__global__ void __launch_bounds__(NT) back_run_all_kernel(const BackArgs a) {
+    back_run_body<EPI, TQ, GENPOT, NT>(a, a.t0 + (int)blockIdx.y, blockIdx.x);
 }
 
 // Persistent batched back projection + update: a resident grid whose blocks
@@ -238,11 +239,11 @@ struct TileBack {
     //   300^2's 361 tiles 8.1 (7.4).
     pet_status run_plain(dim3 grid) const {
         const int blocks = (int)(grid.x * grid.y), sms = sm_count();
-        if (blocks <= sms && max_views > 64) return run_launch<back_run_plain_kernel<1024>, 1024>(grid);
+        if (blocks <= sms && max_views > 64) return run_launch<back_run_all_kernel<EPI_PLAIN, float, false, 1024>, 1024>(grid);
         if (blocks <= 2 * sms) return run_launch<back_run_kernel<EPI_PLAIN, float, false, 512>, 512>(grid);
         if (blocks > 3 * sms && max_views <= 8)
             return run_launch<back_run_kernel<EPI_PLAIN, float, false, kBlock>, kBlock>(grid);
-        return run_launch<back_run_plain_kernel<512>, 512>(grid);
+        return run_launch<back_run_all_kernel<EPI_PLAIN, float, false, 512>, 512>(grid);
     }
 
     template <int EPI, typename TQ, bool GENPOT>
@@ -252,7 +253,16 @@ struct TileBack {
         if constexpr (EPI == EPI_PLAIN) {
             return run_plain(grid);
         } else if constexpr (EPI == EPI_ANCHOR || EPI == EPI_SAGA_INIT || EPI == EPI_SAGAEM_INIT) {
-            return run_launch<back_run_kernel<EPI, TQ, GENPOT, kBlock>, kBlock>(grid);
+            // A table fill takes five blocks an SM (48 registers) unless six spare a
+            // round of blocks or there are many rounds: 64^2 x 6 subsets 18.9 us (six:
+            // 20.6), 201^2 x 7 53.3 (54.8); 256^2 x 3 80.3 (76.1), x 21 80.2 (78.6).
+            if constexpr (EPI == EPI_SAGA_INIT) {
+                const int blocks = tiles * ny_grid, sms = sm_count();
+                const int rounds5 = (blocks + 5 * sms - 1) / (5 * sms), rounds6 = (blocks + 6 * sms - 1) / (6 * sms);
+                if (rounds5 == rounds6 && blocks <= 8 * sms)
+                    return run_launch<back_run_kernel<EPI, TQ, GENPOT, kBlock>, kBlock>(grid);
+            }
+            return run_launch<back_run_all_kernel<EPI, TQ, GENPOT, kBlock>, kBlock>(grid);
         } else {
             if (update_by_runs(a, tiles, max_views)) {
                 const int sms = sm_count();
