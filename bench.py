@@ -60,7 +60,7 @@ def parse_args():
     ap.add_argument("--workload", default="c256")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--recon", type=int, default=200, help="reconstructions per method for the gap metric")
-    ap.add_argument("--tuning", default="", help="pin launch shapes 'chunks,run' instead of autotuning")
+    ap.add_argument("--tuning", default="", help="pin launch shapes 'chunks,run' instead of autotuning (run, 4 or 8, shapes no launch)")
     ap.add_argument("--requests", type=int, default=1000, help="serve workload: number of requests")
     ap.add_argument("--rate", type=float, default=200.0, help="serve workload: mean arrivals per second")
     ap.add_argument("--budget-gib", type=float, default=1.0, help="serve workload: device-memory budget")
@@ -794,8 +794,7 @@ def run_ours(args):
         "vs_baseline": None, "dtype": "f32", "data": "synthetic (seeded ellipse phantom, Poisson counts)",
         "config": dict(workload_config(work, E), parallelism=f"replicas x{world}",
                        concurrency="one batch (pet_batch_epoch)" if args.batch else "four streams",
-                       launch_shapes={"forward_band_chunks": tuning[0], "back_run_pixels": tuning[1],
-                                      "source": tune_src}),
+                       launch_shapes={"forward_band_chunks": tuning[0], "source": tune_src}),
         "p50_ms": float(np.percentile(step_ms, 50)), "p99_ms": float(np.percentile(step_ms, 99)),
         "pairs_per_step": pairs / args.steps,
         "gpu_launches": int(launches),

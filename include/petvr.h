@@ -143,7 +143,8 @@ pet_status pet_plan_nnz(const pet_plan *plan, int32_t t, int64_t *h_nnz);
 /* Launch shapes of the single-slice kernels: band chunks per ray in the
  * forward projector (8, 16 or 32; 0 = size-based default) and back_run (4 or
  * 8), which is kept and reported but shapes no launch: the back projector
- * takes pixels one by one.  The chunk count is the one of subset
+ * stages bins or walks runs of 8 pixels, by the bins per pixel, the views and
+ * the image size.  The chunk count is the one of subset
  * projections; full-data forward passes (objectives, anchor ratios, all-view
  * projections) of images large enough to fill the GPU several times over use
  * half as many, but not fewer than 16.  Results are identical up to the FP32
@@ -155,8 +156,7 @@ pet_status pet_plan_get_tuning(const pet_plan *plan, int32_t *h_fwd_chunks, int3
 /* Autotuner: times every forward chunk count on this plan's own geometry (all
  * subsets, best of three passes on a private stream, synchronising), keeps
  * the fastest, and reports it and back_run (either pointer may be NULL).
- * Allocates and frees scratch images.  Slice
- * stacks have nothing to tune. */
+ * Allocates and frees scratch images.  Slice stacks have nothing to tune. */
 pet_status pet_plan_autotune(pet_plan *plan, int32_t *h_fwd_chunks, int32_t *h_back_run);
 
 /* Device bytes a plan holds, and the bytes pet_problem_create would

@@ -939,7 +939,7 @@ pet_status enqueue_update(pet_state *st, int algo, const int *t_dev, const float
         b.B = st->B;
     } else if (algo == PET_ALGO_SAGA) {
         epi = EPI_SAGA;
-            b.d = st->precond == PET_PRECOND_ITERATE ? nullptr : st->d;
+        b.d = st->precond == PET_PRECOND_ITERATE ? nullptr : st->d;
         b.table = st->table;
         b.qbar = st->qbar;
     } else if (algo == PET_ALGO_SVRG) {
@@ -1917,8 +1917,7 @@ void build_batch_phases(pet_batch *b, int n_iter, const std::vector<std::vector<
                 fa.push_back({j, WK_FWD_ANCHOR, 0, forward_blocks(pl->M, 1, full_group(pl)), full_group(pl), 0});
             }
             const int sub = choose_group(pl);
-            fu.push_back({j, WK_FWD_UPDATE, 0, forward_blocks(max_sub_rays(pl), 1, sub),
-                          sub, 0});
+            fu.push_back({j, WK_FWD_UPDATE, 0, forward_blocks(max_sub_rays(pl), 1, sub), sub, 0});
         }
         // bands per chunk decide an item's length
         auto longer_fwd = [&](const WorkSeg &x, const WorkSeg &y) {
@@ -1993,8 +1992,7 @@ void build_batch_dataflow(pet_batch *b, int n_iter, const std::vector<std::vecto
                 if (st->algo == PET_ALGO_SVREM) ready = true;
             }
             const int sub = choose_group(pl);
-            const int f = add(DF_FWD_UPDATE, forward_blocks(max_sub_rays(pl), 1, sub),
-                              sub, i, 0, prev_b, -1);
+            const int f = add(DF_FWD_UPDATE, forward_blocks(max_sub_rays(pl), 1, sub), sub, i, 0, prev_b, -1);
             prev_b = add(DF_BACK_UPDATE, tiles, 0, i, 0, f, fin);
         }
     }

@@ -3,14 +3,14 @@
 //
 // b_n = sum_{m in S_t} a_mn r_m as a gather per pixel (no atomics, so the
 // result is deterministic).  Single slices use tiles that stage the bins they
-// need of every view (back_tile_kernel, here); slice stacks
-// and multi-ring volumes have their own kernels in volume_back.cu (z-lanes
-// over a pixel's slices; each band piece split over the layers its axial
-// range crosses).  In each view only the bins whose ray
-// can cross the pixel's major band at the pixel are candidates (usually
-// 2-3), found from the bin spacing K, and each candidate's weight comes from
-// band_point() / band_split(), the functions the forward kernels use, so A^T
-// here is the exact transpose of A there.
+// need of every view (back_tile_kernel, here) or walk runs of 8 pixels
+// (back_run_kernel), with the same bits; slice stacks and multi-ring volumes
+// have their own kernels in volume_back.cu (a lane per slice of a pixel; each
+// band piece split over the layers its axial range crosses).  In each view only
+// the bins whose ray can cross the pixel's major band at the pixel are
+// candidates (usually 2-3), found from the bin spacing K, and each candidate's
+// weight comes from band_point() / band_weights(), the functions the forward
+// kernels use, so A^T here is the exact transpose of A there.
 //
 // The epilogue then applies the method's update with b_n still in a
 // register (the penalty's neighbours, 4 in a plane and 2 more along z in a

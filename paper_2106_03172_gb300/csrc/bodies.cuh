@@ -283,9 +283,9 @@ __device__ __forceinline__ void stage_bins(int nq, int bw, Load &&load) {
 // arrive in one, and the views' chains overlap.  The weights are band_weights()
 // of the positions the forward computes, bit for bit (the ends come in order,
 // so the floor, the share and the test of the upper end are all there is to a
-// candidate).  Against runs of 8 pixels a thread (back_run_body), same bound on the
-// blocks per SM: a 201x147 SVRG run 418 -> 373 us, a 512^2 reconstruction 3400 ->
-// 3131, a 256^2 SAGA epoch 163 -> 160, two SVREM epochs 522 -> 534.
+// candidate).  Against runs (back_run_body) as the updates had them before: a
+// 256^2 SAGA epoch of 21 updates 190 -> 162 us, a 201x147 SVRG run 474 -> 381, a 512^2
+// reconstruction 3924 -> 3160; update_by_runs has the points where runs win.
 template <int EPI, typename TQ, bool GENPOT, bool COH = false>
 __device__ __forceinline__ void back_tile_body(const BackArgs &a, const int t, const int bx) {
     constexpr int NT = kTile * kTile;
@@ -404,7 +404,8 @@ __device__ __forceinline__ void back_tile_body(const BackArgs &a, const int t, c
     }
 }
 
-// All-subset launches (anchors, table fills) and plain back projections: for each
+// All-subset launches (anchors, table fills), plain back projections, and the updates
+// and batch members that are faster this way (update_by_runs, batch_runs): for each
 // view, the tile's bands are cut into runs of kRun pixels along the view's minor
 // axis; one thread walks the rays that can cross a run in order and adds each
 // ray's two band pieces into per-view partial sums in shared memory (every
