@@ -112,3 +112,20 @@ def test_update_shapes_have_the_same_bits(mode, nx, ny, per_subset, fineness):
         batch.epoch([[1, 0, 1]], [alpha], [1])
         batch.sync()
         assert torch.equal(alone, batched), method
+
+
+# launches whose subset is given by the host: the warm start's updates and SEM's statistic of all views
+@pytest.mark.parametrize("nx,ny,per_subset,fineness", [
+    (40, 37, 7, 1.0), (40, 37, 11, 0.77), (40, 37, 6, 4.0), (120, 90, 13, 1.6), (120, 90, 9, 4.0)])
+def test_warm_start_and_sem_shapes(nx, ny, per_subset, fineness):
+    from paper_2106_03172_gb300 import petvr as pv
+    geom, g = _update_problem(nx, ny, per_subset, fineness)
+    prob = em.build_problem(geom, g.astype(np.float64), 0.5, 2, 0.01)
+    plan = pv.Plan(geom, 2)
+    gp = pv.Problem(plan, _cuda(g), None, 0.5, 0.01)
+    img = torch.empty(prob.N, device="cuda")
+    pv.pet_warm_start(gp.handle, img)
+    f0 = _host(img).reshape(-1, 1)
+    assert rel_l2(f0, prob.initial_image()) <= 1e-5
+    pv.State(gp, "sem", img).epoch([1], alpha=0.5)
+    assert rel_l2(_host(img), em.SEM(prob, f0, schedule=lambda k: 0.5).step(1)) <= 1e-5
